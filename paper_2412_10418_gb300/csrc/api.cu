@@ -521,7 +521,7 @@ void forward(cdsl_ctx* c, ModelW& m, const RowDesc* rows, int R, int lm_rows,
     at.qb_count = (ap.rows_per_prompt * at.G + at.qblock - 1) / at.qblock;
     n_z = c->B * at.qb_count;
   }
-  const int ld_ss = c->R_pad;
+  const int ld_ss = c->d_max / 32;
   auto normed_input = [&](GemmArgs& a, const float* ss) {
     a.in_ss = ss; a.norm_D = D; a.ld_ss = ld_ss; a.norm_eps = cfg.norm_eps;
   };
@@ -618,7 +618,7 @@ void do_verify(cdsl_ctx* c) {
   a.next_x = c->st.x; a.amax = c->st.v_amax; a.logp = c->st.v_logp; a.topk = c->st.v_topk;
   a.status = c->st.status;
   if (c->run.reward_head) {
-    a.ss = c->ss_a; a.hw = c->ss_hw; a.norm_D = c->tcfg.d_model; a.ld_ss = c->R_pad;
+    a.ss = c->ss_a; a.hw = c->ss_hw; a.norm_D = c->tcfg.d_model; a.ld_ss = c->d_max / 32;
     a.norm_eps = c->tcfg.norm_eps; a.head_out = c->st.v_head;
   }
   timed(c, K_ROWSTATS, 0, 0, [&] {
@@ -661,7 +661,7 @@ void do_step1_round(cdsl_ctx* c) {
       launch_row_stats(a, c->stream);
     });
   timed(c, K_STEPLOGIC, 0, 0, [&] {
-    launch_select_s1(c->st, c->tgt.kv, c->dft.kv, c->ss_a, c->ss_hw, c->tcfg.d_model, c->R_pad,
+    launch_select_s1(c->st, c->tgt.kv, c->dft.kv, c->ss_a, c->ss_hw, c->tcfg.d_model, c->d_max / 32,
                      c->tcfg.norm_eps, c->stream);
   });
 }

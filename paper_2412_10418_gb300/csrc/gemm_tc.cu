@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int R = min(a.R, NP);
     if (a.in_ss || (kBig && a.mode == EPI_QKV)) {   // once per block, while the first
       if (a.in_ss) input_row_scales(a, 0, R, s_rs, etid, kEpThreads);   // accumulator fills
-      if (kBig && a.mode == EPI_QKV) qkv_rows(a, R, s_qkv, etid, kEpThreads);
+      if (kBig && a.mode == EPI_QKV) qkv_rows(a, 0, R, s_qkv, etid, kEpThreads);
       tc::named_barrier(1, kEpThreads);
     }
     while (u < u1) {

@@ -56,7 +56,7 @@ __global__ void k_embed(const RowDesc* rows, const T* E, int D, float* h, T* x, 
       store_act<T>(x, plane, (size_t)r * D + c, v * to_f32<T>(g[c]));
     }
     const float sq = warp_sum(v * v);
-    if ((threadIdx.x & 31) == 0 && c < D) ss[(size_t)(c >> 5) * ld_ss + r] = sq;
+    if ((threadIdx.x & 31) == 0 && c < D) ss[(size_t)r * ld_ss + (c >> 5)] = sq;
   }
 }
 
@@ -169,12 +169,10 @@ __global__ void __launch_bounds__(RS_THREADS) k_row_stats(RowStatsArgs a) {
   if (a.amax && threadIdx.x == 0) a.amax[r] = amax;
   if (a.head_out && threadIdx.x < 32) {   // sigmoid(w . g . h * row scale) from the partials
     float hw = 0.f;
-    for (int c = threadIdx.x; c < (a.norm_D >> 5); c += 32) hw += a.hw[(size_t)c * a.ld_ss + r];
+    for (int c = threadIdx.x; c < (a.norm_D >> 5); c += 32) hw += a.hw[(size_t)r * a.ld_ss + c];
     hw = warp_sum(hw);
-    if (threadIdx.x == 0) {
-      const float rs = row_scale(a.ss, a.norm_D >> 5, a.ld_ss, r, a.norm_D, a.norm_eps);
-      a.head_out[r] = 1.0f / (1.0f + expf(-hw * rs));
-    }
+    const float rs = row_scale(a.ss, a.norm_D >> 5, a.ld_ss, r, a.norm_D, a.norm_eps);
+    if (threadIdx.x == 0) a.head_out[r] = 1.0f / (1.0f + expf(-hw * rs));
   }
   if (a.dp1 > 0 && threadIdx.x == 0) {
     const int j = r % a.dp1, bi = r / a.dp1, d = a.dp1 - 1;
@@ -490,7 +488,7 @@ __global__ void k_select_s1(StepState st, KvStore tkv, KvStore dkv, const float*
   if (st.reward_head) {
     const int row = 2 * st.B + b * d + d - 1;   // lh_d
     float h = 0.f;
-    for (int c = lane; c < (norm_D >> 5); c += 32) h += hw[(size_t)c * ld_ss + row];
+    for (int c = lane; c < (norm_D >> 5); c += 32) h += hw[(size_t)row * ld_ss + c];
     h = warp_sum(h);
     const float rs = row_scale(ss, norm_D >> 5, ld_ss, row, norm_D, eps);
     r = 0.5f * cov + 0.5f * (1.0f / (1.0f + expf(-h * rs)));

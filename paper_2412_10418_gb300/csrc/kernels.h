@@ -184,7 +184,7 @@ void launch_plan_s1_verify(const StepState& st, RowDesc* rows, cudaStream_t s);
 // commit = 0: decide only (n_b, rewards, b*, state, emission); 1: also allocate KV pages
 void launch_select(const StepState& st, KvStore tkv, KvStore dkv, int commit, cudaStream_t s);
 // Step-1 round 2's decision: R(T + c_1 + x' + lh) >= r_t emits c_1, x' (state 3). ss / hw:
-// the target pass's final-norm and reward-head partial sums (ld_ss rows apart).
+// the target pass's final-norm and reward-head partial sums (rows ld_ss apart).
 void launch_select_s1(const StepState& st, KvStore tkv, KvStore dkv, const float* ss,
                       const float* hw, int norm_D, int ld_ss, float norm_eps, cudaStream_t s);
 void launch_commit_kv(const StepState& st, KvStore kv, int slots_per_beam, int is_draft,
