@@ -77,7 +77,7 @@ struct cdsl_ctx {
   int32_t* lm_gather = nullptr;
   int32_t* lm_dst = nullptr;
   float* gemv_part = nullptr;   // split-K partial tiles of the weight-streaming GEMM
-  int32_t* gemv_cnt = nullptr;  // per-tile arrival counters, then per-tile finished shares
+  int32_t* gemv_cnt = nullptr;  // per-tile arrival counters
   int plan_sms = kPlanSMs;      // SMs the tensor-core GEMM plans for: min(kPlanSMs, device's)
   int32_t* attn_zmap = nullptr; // prefill: z -> (prompt, query block)
   int attn_zmax = 0, attn_chunks = 0;
@@ -286,7 +286,7 @@ size_t carve(cdsl_ctx* c, void* base) {
         part = std::max(part, (size_t)p.splits * 8 * p.tiles * 128);
         tiles = std::max(tiles, (size_t)p.tiles);
         if (c->dtype == CDSL_DTYPE_BF16 && sh[0] % 64 == 0) {
-          for (int R = 9; R <= std::min(c->R_max, 256); R += 16) {  // every n_pad in use
+          for (int R = 9; R <= std::min(c->R_max, kPairRows); R += 16) {  // every n_pad in use
             // the plan, and stream-K, which a plan falls back to where clusters do not fit
             const TcPlan t = plan_tc(sh[0], sh[1], R, kPlanSMs);
             const TcPlan sk = plan_tc(sh[0], sh[1], R, kPlanSMs, 0, 0, 0);
@@ -297,7 +297,7 @@ size_t carve(cdsl_ctx* c, void* base) {
       }
     }
     c->gemv_part = cv.take<float>(part);
-    c->gemv_cnt = cv.take<int32_t>(2 * tiles);
+    c->gemv_cnt = cv.take<int32_t>(tiles);
   }
   {  // attention: the prefill's (prompt, query block) map
     const int QB = attn_qblock();
@@ -417,19 +417,27 @@ void gemm(cdsl_ctx* c, const GemmArgs& a) {
       launch_gemv(as, plan_gemv(a.K, a.n_virtual, kPlanSMs), c->gemv_part, c->gemv_cnt, c->stream);
     });
   } else if (impl == K_GEMM_TC) {
+    // more than kPairRows rows: pairs of SMs (gemm_pair.cu)
+    const bool pair = a.R > kPairRows;
+    const TcPlan p = pair ? TcPlan{} : plan_tc(a.K, a.n_virtual, a.R, c->plan_sms);
+    const PairPlan pp =
+        pair ? plan_pair(a.mode, a.K, a.n_virtual, a.R, c->plan_sms) : PairPlan{};
     TcMaps maps;
     for (int s = 0; s < 3; ++s) {
       const int seg = s < a.n_seg ? s : 0;
-      maps.w[s] = tensor_map(c, a.w[seg], a.K, a.seg_rows[seg], 64);
+      maps.w[s] = tensor_map(c, a.w[seg], a.K, a.seg_rows[seg],
+                             pair ? pair_box_rows(a.mode, a.kv.hd) : 64);
     }
     const __nv_bfloat16* xb = reinterpret_cast<const __nv_bfloat16*>(a.x);
-    const TcPlan p = plan_tc(a.K, a.n_virtual, a.R, c->plan_sms);
-    // activation boxes: 64 features x n_pad rows (<= 256 <= R_pad), one per plane and stage
-    maps.xh = tensor_map(c, xb, a.ldx, c->R_pad, p.n_pad);
-    maps.xl = tensor_map(c, xb + a.x_plane, a.ldx, c->R_pad, p.n_pad);
+    // activation boxes: 64 features x the tile's rows (a pair's CTAs load half each), one per
+    // plane and stage
+    const int box = pair ? pp.n / 2 : p.n_pad;
+    maps.xh = tensor_map(c, xb, a.ldx, c->R_pad, box);
+    maps.xl = tensor_map(c, xb + a.x_plane, a.ldx, c->R_pad, box);
     timed(c, impl, by, fl, [&] {
       as.stamp = c->cur_stamp;
-      launch_gemm_tc(maps, as, p, c->gemv_part, c->gemv_cnt, c->stream);
+      if (pair) launch_gemm_pair(maps, as, pp, c->stream);
+      else launch_gemm_tc(maps, as, p, c->gemv_part, c->gemv_cnt, c->stream);
     });
   } else {
     timed(c, impl, by, fl, [&] {
@@ -795,7 +803,11 @@ int32_t cdsl_init(const cdsl_model_cfg* target, const void* const* h_target_weig
     delete c;
     return fail(nullptr, CDSL_ECUDA, "cannot configure the tensor-core GEMM (shared memory)");
   }
-  {  // the large-row GEMM's stream-K grid must be resident at once (one block per SM)
+  if (c->dtype == CDSL_DTYPE_BF16 && configure_gemm_pair()) {
+    delete c;
+    return fail(nullptr, CDSL_ECUDA, "cannot configure the paired tensor-core GEMM");
+  }
+  {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)

@@ -148,7 +148,7 @@ constexpr int kPlanSMs = 152;  // GB300: split-K is planned for this many SMs
 GemvPlan plan_gemv(int K, int n_virtual, int n_sm);
 void launch_gemv(const GemmArgs& a, const GemvPlan& p, float* part, int* tile_cnt, cudaStream_t s);
 
-// Tensor-core GEMM (tcgen05, TMEM, TMA) for bf16 weights and 1..256 activation rows, on a
+// Tensor-core GEMM (tcgen05, TMEM, TMA) for bf16 weights and 1..kPairRows activation rows, on a
 // persistent stream-K grid of `ctas` blocks. maps: TMA descriptors of the weight segments
 // (128-byte swizzle, 64x64 boxes) and of the hi / lo activation planes (64x16 boxes).
 // Scratch: part [ctas][2][n_pad][128] floats (tc_scratch_floats), one arrival counter per
@@ -156,8 +156,7 @@ void launch_gemv(const GemmArgs& a, const GemvPlan& p, float* part, int* tile_cn
 struct TcMaps { CUtensorMap w[3]; CUtensorMap xh, xl; };
 // cluster > 0: cluster split-K with that many blocks per tile (ctas = tiles * cluster); 0:
 // persistent stream-K over ctas blocks.
-// big: the variant for more than 64 activation rows (k_gemm_tc<true>)
-struct TcPlan { int tiles, kb_total, ctas, n_pad, stages, ep_rows, cluster, big; size_t smem; };
+struct TcPlan { int tiles, kb_total, ctas, n_pad, stages, ep_rows, cluster; size_t smem; };
 bool tc_supported(const GemmArgs& a);
 // cluster: -1 chooses (split-K clusters when every tile fits at once with >= 2 blocks), 0
 // stream-K, > 0 that cluster size.
@@ -169,6 +168,20 @@ int encode_bf16_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t o
 int configure_gemm_tc();
 void launch_gemm_tc(const TcMaps& maps, const GemmArgs& a, const TcPlan& p, float* part,
                     int* tile_cnt, cudaStream_t s);
+
+// The same projections for more than kPairRows activation rows, on pairs of SMs (gemm_pair.cu):
+// tiles of 256 weight rows (times two accumulators for QKV and gate/up) x n activation rows.
+// maps: weight boxes of 64 features x pair_box_rows() rows, activation boxes of 64 x n / 2.
+// n_tiles tiles of n rows cover the pass; split: pairs per cluster sharing a tile's K range;
+// bufs: accumulator sets in TMEM; seg: a tile's K range in several accumulation chains; planes:
+// 2 where hi and lo accumulate apart. No scratch.
+constexpr int kPairRows = 64;
+struct PairPlan { int n, n_tiles, m_tiles, kb_total, split, stages, bufs, seg, planes, ctas; size_t smem; };
+PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt = 0,
+                   int force_split = 0);
+int pair_box_rows(int mode, int hd);
+int configure_gemm_pair();
+void launch_gemm_pair(const TcMaps& maps, const GemmArgs& a, const PairPlan& p, cudaStream_t s);
 
 // Message returned by cdsl_last_error(NULL) on this thread.
 void set_thread_error(const char* msg);
