@@ -214,10 +214,12 @@ void derive_dims(cdsl_ctx* c) {
   c->R_d = c->B * c->k + c->B;
   // Step-1 round 2: the target pass holds d+2 rows per prompt (draft calls fit in R_d)
   c->R_s1 = r.step1_budget >= 2 ? c->B * (c->d + 2) : 0;
-  // default 256 prefill rows (the most the tensor-core GEMM takes): the large-row GEMM then
-  // streams each weight once per 256 prompt tokens (measured, 512-token 7B prefill: 43 ms at
-  // 64 rows, 35 at 128, 33 at 256; 13B, 4 x 1024 tokens: 564, 464, 428 ms)
-  const int chunk = r.max_chunk ? r.max_chunk : 256;
+  // default 1024 prefill rows: the paired GEMM then has several row tiles per weight tile, each
+  // weight is streamed once per 1024 prompt tokens, and a pass's launches and the wait that ends
+  // it are shared by as many tokens (measured, prefill and first step: 32 small-model prompts
+  // 14.3 ms at 256 rows, 9.7 at 512, 7.5 at 1024, 6.6 at 2048; 13B two-layer, 3,500 tokens
+  // 19.8, 17.6, 15.2, 13.7; the activation buffers grow with it, 170 MB of a 13B workspace)
+  const int chunk = r.max_chunk ? r.max_chunk : 1024;
   c->R_p = std::min(chunk, c->B * r.max_prompt);
   c->R_max = std::max(std::max(c->R_v, c->R_s1), std::max(c->R_d, c->R_p));
   c->R_pad = (c->R_max + 31) / 32 * 32;
