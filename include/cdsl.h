@@ -249,20 +249,13 @@ CDSL_API int32_t cdsl_get_status(cdsl_ctx* ctx, int32_t* h_device_status);
  * callers of this library that cannot allocate device memory: host frameworks whose own
  * caching allocator has already reserved the GPU's memory, real-time loops that must not
  * block on cudaMalloc / cudaFree, and runtimes that forbid device allocation after start-up.
- * y[R, N] = x[R, K] W^T with fp32 accumulation, computed by the library's CUDA-core split-K
- * GEMV (x is split into bf16 hi and lo planes, so the result is within about 1e-5 relative
- * of the exact product): d_w [N, K] bfloat16 row-major, d_x [R, K] float32, d_y [R, N]
- * float32, all device pointers on the current device, contiguous and 16-byte aligned; stream
- * is a cudaStream_t (NULL: the legacy stream).
+ * y[R, N] = x[R, K] W^T with fp32 products and sums on the CUDA cores: d_w [N, K] bfloat16
+ * row-major, d_x [R, K] float32, d_y [R, N] float32, all device pointers on the current device,
+ * contiguous and 16-byte aligned; stream is a cudaStream_t (NULL: the legacy stream).
  * Limits: 1 <= R <= 8, 8 <= K <= 8192 with K % 8 == 0, 1 <= N <= 32768; anything beyond them
- * returns CDSL_EINVAL without launching. Its scratch (split-K partials, arrival counters and
- * the hi/lo activation planes, 8.3 MiB) is one fixed array inside the library, which every
- * GPU that loads the library holds until the process exits; no call allocates or frees.
- * Set-up: the first call in each CUDA context looks up that array's device address (and
- * clears its counters) with the context current. Only contexts that stay alive are
- * supported: after a device reset the array's address may be stale. Every call shares the
- * array: calls that overlap on a GPU (other streams or threads) race, and the caller must
- * order them. Asynchronous on `stream`; errors via cdsl_last_error(NULL). */
+ * returns CDSL_EINVAL without launching. One kernel without scratch in global memory: no call
+ * allocates or frees, and calls on other streams or threads may overlap. Asynchronous on
+ * `stream`; errors via cdsl_last_error(NULL). */
 CDSL_API int32_t cdsl_gemv_noalloc(const void* d_w, int32_t N, int32_t K, const float* d_x,
                                    int32_t R, float* d_y, void* stream);
 
