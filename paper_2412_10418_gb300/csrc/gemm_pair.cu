@@ -21,9 +21,11 @@
 // most kSegKb blocks (2.2e-6), into two TMEM accumulator sets in turn; the epilogue warps add each
 // finished segment to fp32 sums in their registers (rounded to nearest) while the next one
 // accumulates (k_gemm_pair<.., true>). A K range of one segment is finished straight from TMEM
-// (<.., false>), and so are QKV and gate/up tiles of more than 128 rows, whose two accumulators
-// leave TMEM no room for a second set: one chain, for K up to kWideKb blocks. Where TMEM has
-// room (planes == 2) the lo plane accumulates apart, which halves a chain's truncations.
+// (<.., false>), and so are gate/up tiles of more than 128 rows, whose two accumulators leave
+// TMEM no room for a second set: one chain, for K up to kWideKb blocks (13B gate/up, 224 rows: 88
+// us against 115; the kernel before had the same chain there). Where TMEM has room (planes == 2)
+// the lo plane accumulates apart, which halves a chain's truncations. 13B logits after two layers,
+// against 64 bits: 2.1e-5 (the kernel before: 2.7e-5; one chain per tile in all shapes: 3.3e-5).
 //
 // Schedule (plan_pair): the tiles of a launch are dealt to the pairs in turn (persistent), or,
 // with few tiles, a cluster of S pairs splits a tile's K range: the partial tiles go to shared
@@ -621,8 +623,9 @@ PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt
       // chain where the tile's accumulators leave TMEM no room for it
       const int nkb = (KBT + S - 1) / S;
       const bool wide = MT * N > 256, seg = nkb > kSegKb && !wide;
-      if (wide && nkb > kWideKb) continue;
-      const int bufs = wide || (!seg && waves == 1) ? 1 : 2;
+      if (wide && (mode != EPI_SWIGLU || nkb <= kSegKb || nkb > kWideKb)) continue;
+      // short chains keep lo apart rather than a second set where TMEM has no room for both
+      const int bufs = wide || (!seg && (waves == 1 || 4 * MT * N > 512)) ? 1 : 2;
       const int stages = (int)std::min<size_t>(kStagesMax, (kSmemMax - 1024) / stage);
       if (S > 1 && (size_t)stages * stage < (size_t)MT * N * 512) continue;
       const int planes = 2 * bufs * MT * N <= 512 ? 2 : 1;
