@@ -477,19 +477,24 @@ const CUtensorMap& tensor_map(cdsl_ctx* c, const void* base, int inner, int oute
   return c->maps.emplace(key, m).first->second;
 }
 
-// Query vectors per prompt and KV head from which a dense pass of a bf16 model runs on the
-// tensor-core attention (attention_tc.cu) rather than the CUDA-core one (attention.cu). The
-// 7B verify pass (80) measured 16.3 us per launch on the former against 20.1 us on the
-// latter; decode passes (16-36) stay on the CUDA cores, where a block's 64-key chunk is too
-// small for the MMA's 128 rows to pay.
+// Query vectors per prompt and KV head from which a pass of a bf16 model runs on the tensor-core
+// attention (attention_tc.cu) rather than the CUDA-core one (attention.cu). The 7B verify pass
+// (80) measured 16.3 us per launch on the former against 20.1 us on the latter; decode passes
+// (16-36) stay on the CUDA cores, where a block's 64-key chunk is too small for the MMA's 128 rows
+// to pay.
 constexpr int kAttnTcMinVectors = 64;
+bool use_attn_tc(const cdsl_ctx* c, int rows_per_prompt, int G) {
+  return c->dtype == CDSL_DTYPE_BF16 && rows_per_prompt * G >= kAttnTcMinVectors;
+}
 
 // One forward pass of a model over R rows described by `rows`; for lm_rows > 0 the final
 // norm + LM head run over rows gather[i] (or the first lm_rows rows) into logits.
 // Attention layout of a pass: rows per prompt (dense z mapping) or a host-built z map.
 struct AttnPass {
-  int rows_per_prompt = 0;            // dense: z = b * qb_count + qb
-  const std::vector<int32_t>* zmap = nullptr;  // prefill: (b, qb) pairs for this model
+  int rows_per_prompt = 0;            // dense: z = b * qb_count + qb; prefill: of the prompt
+                                      //   with the most rows
+  const std::vector<int32_t>* zmap = nullptr;  // prefill: (b, qb) pairs for this model, in
+  int qblock = 0;                              //   query blocks of qblock vectors
   int n_chunks = 0;
   int n_tchunks = 0;                  // tail-key chunks (attn_tail_chunks)
 };
@@ -513,21 +518,15 @@ void forward(cdsl_ctx* c, ModelW& m, const RowDesc* rows, int R, int lm_rows,
   at.status = c->st.status;
   at.wait_ns = c->wait_ns;
   int n_z;
-  // dense passes of bf16 models with many query vectors per KV head on the tensor-core
-  // attention (kAttnTcMinVectors)
-  const bool attn_tc = c->dtype == CDSL_DTYPE_BF16 && !ap.zmap &&
-                       ap.rows_per_prompt * (H / KVH) >= kAttnTcMinVectors;
-  if (attn_tc) {
-    at.qblock = attn_tc_qblock(ap.rows_per_prompt, at.G);
-    at.qb_count = (ap.rows_per_prompt * at.G + at.qblock - 1) / at.qblock;
-    n_z = c->B * at.qb_count;
-  } else if (ap.zmap) {
+  const bool attn_tc = use_attn_tc(c, ap.rows_per_prompt, at.G);
+  if (ap.zmap) {
     n_z = (int)ap.zmap->size() / 2;
     at.zmap = c->attn_zmap;
-    at.qblock = attn_qblock();
+    at.qblock = ap.qblock;
     cudaMemcpyAsync(c->attn_zmap, ap.zmap->data(), ap.zmap->size() * 4, cudaMemcpyHostToDevice, s);
   } else {
-    at.qblock = attn_qblock_for(ap.rows_per_prompt, at.G);
+    at.qblock = attn_tc ? attn_tc_qblock(ap.rows_per_prompt, at.G, ap.n_tchunks > 0)
+                        : attn_qblock_for(ap.rows_per_prompt, at.G);
     at.qb_count = (ap.rows_per_prompt * at.G + at.qblock - 1) / at.qblock;
     n_z = c->B * at.qb_count;
   }
@@ -877,18 +876,22 @@ int32_t cdsl_prefill(cdsl_ctx* c, const int32_t* d_prompts, const int32_t* h_pro
     std::vector<int> per_prompt(B, 0);
     int maxpos = 0;
     for (const RowDesc& rd : rows) { per_prompt[rd.b]++; maxpos = std::max(maxpos, rd.pos); }
-    auto zmap_for = [&](const cdsl_model_cfg& mc) {
+    const int most = *std::max_element(per_prompt.begin(), per_prompt.end());
+    auto zmap_for = [&](const cdsl_model_cfg& mc, AttnPass* ap) {
       std::vector<int32_t> z;
-      const int G = mc.n_heads / mc.n_kv_heads;
+      const int G = group_size(mc);
+      ap->rows_per_prompt = most;
+      ap->qblock = use_attn_tc(c, most, G) ? attn_tc_qblock(most, G, false) : attn_qblock();
+      // a prompt's last query blocks, which see the most keys, first
       for (int b = 0; b < B; ++b)
-        for (int q = 0; q < (per_prompt[b] * G + attn_qblock() - 1) / attn_qblock(); ++q) {
+        for (int q = (per_prompt[b] * G + ap->qblock - 1) / ap->qblock - 1; q >= 0; --q) {
           z.push_back(b);
           z.push_back(q);
         }
       return z;
     };
-    const std::vector<int32_t> zt = zmap_for(c->tcfg), zd = zmap_for(c->dcfg);
     AttnPass apt, apd;
+    const std::vector<int32_t> zt = zmap_for(c->tcfg, &apt), zd = zmap_for(c->dcfg, &apd);
     apt.zmap = &zt;
     apd.zmap = &zd;
     apt.n_chunks = apd.n_chunks = (maxpos + attn_chunk()) / attn_chunk();

@@ -1,4 +1,4 @@
-// attention_tc.cu -- attention of the decode and verify passes of bf16 models on the
+// attention_tc.cu -- attention of the prefill and verify passes of bf16 models on the
 // 5th-generation tensor cores (tcgen05 MMA into TMEM).
 //
 // The pass is split as in attention.cu (attn_layout.cuh): a thread-block cluster of up to 16
@@ -58,7 +58,8 @@ constexpr float kLog2e = 1.44269504088896341f;
 
 int g_tc_max_cluster = 8;
 
-template <int HD>
+// NP: planes of P and V (2: x = hi + lo; 3: hi + mid + lo, fp32's own precision).
+template <int HD, int NP>
 struct TcSmem {
   static constexpr int KB = HD / 64;                        // 64-wide K blocks of Q and K
   static constexpr uint32_t Q_KB = TQB * 128;               // bytes of one K block of Q
@@ -70,8 +71,8 @@ struct TcSmem {
   static constexpr uint32_t Q_OFF = 0;
   static constexpr uint32_t K_OFF = Q_OFF + 2 * Q_PLANE;
   static constexpr uint32_t V_OFF = K_OFF + 2 * K_PLANE;
-  static constexpr uint32_t P_OFF = V_OFF + 2 * V_PLANE;
-  static constexpr uint32_t TOTAL = P_OFF + 2 * P_PLANE;
+  static constexpr uint32_t P_OFF = V_OFF + NP * V_PLANE;
+  static constexpr uint32_t TOTAL = P_OFF + NP * P_PLANE;
   static constexpr int OP = HD + 4;                         // row pitch of the partial o (floats)
   static constexpr uint32_t O_OFF = K_OFF;                  // partial o [128][OP] fp32, after the
   static_assert(TQB * OP * 4 <= TOTAL - K_OFF, "partial o fits over K, V and P");   // chunks
@@ -79,29 +80,35 @@ struct TcSmem {
   static constexpr size_t bytes = TOTAL + 1024;             // + 1024-byte alignment of the base
 };
 
-// 8 fp32 values -> 8 bf16 hi values and 8 bf16 lo values (x = hi + lo to about 2^-17).
-__device__ __forceinline__ void split8(const float (&x)[8], uint4& hi, uint4& lo) {
-  uint32_t h[4], l[4];
+// 8 fp32 values -> NP planes of 8 bf16 values: x = hi + lo to about 2^-17, with three planes to
+// about 2^-25.
+template <int NP>
+__device__ __forceinline__ void split8(const float (&x)[8], uint4 (&p)[NP]) {
+  float r[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(x[2 * i]), h1 = __float2bfloat16_rn(x[2 * i + 1]);
-    const __nv_bfloat16 l0 = __float2bfloat16_rn(x[2 * i] - __bfloat162float(h0));
-    const __nv_bfloat16 l1 = __float2bfloat16_rn(x[2 * i + 1] - __bfloat162float(h1));
-    h[i] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-    l[i] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+  for (int i = 0; i < 8; ++i) r[i] = x[i];
+#pragma unroll
+  for (int n = 0; n < NP; ++n) {
+    uint32_t u[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const __nv_bfloat16 a = __float2bfloat16_rn(r[2 * i]), b = __float2bfloat16_rn(r[2 * i + 1]);
+      u[i] = (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+      r[2 * i] -= __bfloat162float(a);
+      r[2 * i + 1] -= __bfloat162float(b);
+    }
+    p[n] = make_uint4(u[0], u[1], u[2], u[3]);
   }
-  hi = make_uint4(h[0], h[1], h[2], h[3]);
-  lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
 __device__ __forceinline__ void st_shared16(uint8_t* base, uint32_t off, const uint4& v) {
   *reinterpret_cast<uint4*>(base + off) = v;
 }
 
-template <int HD>
+template <int HD, int NP>
 __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
   const LaunchStamp stamp(a.stamp);
-  using SM = TcSmem<HD>;
+  using SM = TcSmem<HD, NP>;
   constexpr int KB = SM::KB;
   constexpr int DCH = HD / 8;                    // 16-byte bf16 chunks per row of Q and K
   constexpr int K_IT = ACH * DCH / TTHREADS;     // staging items per thread: K (key, chunk)
@@ -124,7 +131,8 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
   const int cx = (int)blockIdx.x;                 // = rank in the cluster
   const int g = blockIdx.y;
   const int n_p = a.n_chunks;
-  const int b = blockIdx.z / a.qb_count, qb = blockIdx.z % a.qb_count;
+  const int b = a.zmap ? a.zmap[2 * blockIdx.z] : blockIdx.z / a.qb_count;
+  const int qb = a.zmap ? a.zmap[2 * blockIdx.z + 1] : blockIdx.z % a.qb_count;
   const int G = a.G, H = a.n_heads;
   const int warp = threadIdx.x >> 5;
 
@@ -223,11 +231,11 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
       const float sc = a.scale * kLog2e;
       const float x[8] = {qr[u][0].x * sc, qr[u][0].y * sc, qr[u][0].z * sc, qr[u][0].w * sc,
                           qr[u][1].x * sc, qr[u][1].y * sc, qr[u][1].z * sc, qr[u][1].w * sc};
-      uint4 hi, lo;
-      split8(x, hi, lo);
+      uint4 p[2];
+      split8<2>(x, p);
       const uint32_t off = SM::Q_OFF + (dc >> 3) * SM::Q_KB + tc::sw128_offset(qv, dc & 7);
-      st_shared16(sm, off, hi);
-      st_shared16(sm, off + SM::Q_PLANE, lo);
+      st_shared16(sm, off, p[0]);
+      st_shared16(sm, off + SM::Q_PLANE, p[1]);
     }
   }
 
@@ -244,20 +252,20 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
       const int idx = threadIdx.x + u * TTHREADS, j = idx / DCH, dc = idx % DCH;
       const float x[8] = {kr[u][0].x, kr[u][0].y, kr[u][0].z, kr[u][0].w,
                           kr[u][1].x, kr[u][1].y, kr[u][1].z, kr[u][1].w};
-      uint4 hi, lo;
-      split8(x, hi, lo);
+      uint4 p[2];
+      split8<2>(x, p);
       const uint32_t off = SM::K_OFF + (dc >> 3) * SM::K_KB + tc::sw128_offset(j, dc & 7);
-      st_shared16(sm, off, hi);
-      st_shared16(sm, off + SM::K_PLANE, lo);
+      st_shared16(sm, off, p[0]);
+      st_shared16(sm, off + SM::K_PLANE, p[1]);
     }
 #pragma unroll
     for (int u = 0; u < V_IT; ++u) {
       const int idx = threadIdx.x + u * TTHREADS, d = idx % HD, jc = idx / HD;
-      uint4 hi, lo;
-      split8(vr[u], hi, lo);
+      uint4 p[NP];
+      split8<NP>(vr[u], p);
       const uint32_t off = SM::V_OFF + tc::sw128_offset(d, jc);
-      st_shared16(sm, off, hi);
-      st_shared16(sm, off + SM::V_PLANE, lo);
+#pragma unroll
+      for (int n = 0; n < NP; ++n) st_shared16(sm, off + n * SM::V_PLANE, p[n]);
     }
     tc::fence_proxy_async();
     __syncthreads();
@@ -354,29 +362,34 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
         float x[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) x[e] = s[cc >> 1][(cc & 1) * 8 + e];
-        uint4 hi, lo;
-        split8(x, hi, lo);
+        uint4 p[NP];
+        split8<NP>(x, p);
         const uint32_t off = SM::P_OFF + tc::sw128_offset(qi, 4 * half + cc);
-        st_shared16(sm, off, hi);
-        st_shared16(sm, off + SM::P_PLANE, lo);
+#pragma unroll
+        for (int n = 0; n < NP; ++n) st_shared16(sm, off + n * SM::P_PLANE, p[n]);
       }
       tc::fence_proxy_async();
       tc::tc_fence_before();
     }
     __syncthreads();
-    // ---- O += P V (hi.hi + hi.lo + lo.hi over the chunk's 64 keys)
+    // ---- O += P V over the chunk's 64 keys: hi.hi + hi.lo + lo.hi, or with three planes the six
+    //      products down to 2^-24 of the largest
     if (threadIdx.x == kIssuer) {
       tc::tc_fence_after();
-      const uint64_t ph = tc::desc_sw128(sbase + SM::P_OFF);
-      const uint64_t pl = tc::desc_sw128(sbase + SM::P_OFF + SM::P_PLANE);
-      const uint64_t vh = tc::desc_sw128(sbase + SM::V_OFF);
-      const uint64_t vl = tc::desc_sw128(sbase + SM::V_OFF + SM::V_PLANE);
+      uint64_t pd[NP], vd[NP];
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        tc::umma_bf16(t_o, ph + 2 * kk, vh + 2 * kk, idesc_o, (nproc | kk) ? 1u : 0u);
-        tc::umma_bf16(t_o, ph + 2 * kk, vl + 2 * kk, idesc_o, 1u);
-        tc::umma_bf16(t_o, pl + 2 * kk, vh + 2 * kk, idesc_o, 1u);
+      for (int n = 0; n < NP; ++n) {
+        pd[n] = tc::desc_sw128(sbase + SM::P_OFF + n * SM::P_PLANE);
+        vd[n] = tc::desc_sw128(sbase + SM::V_OFF + n * SM::V_PLANE);
       }
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+        for (int n = 0; n < NP; ++n)
+#pragma unroll
+          for (int m = 0; n + m < NP; ++m)
+            tc::umma_bf16(t_o, pd[n] + 2 * kk, vd[m] + 2 * kk, idesc_o,
+                          (nproc | kk | n | m) ? 1u : 0u);
       tc::umma_commit(&bar_o);
     }
     ++nproc;
@@ -483,49 +496,57 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
   if (warp == 0) tc::tmem_dealloc(tmem, SM::TMEM_COLS);
 }
 
-template <int HD>
-ClusterFit g_tc_fit;   // cluster residency of k_attn_tc<HD> (configure_tc)
+template <int HD, int NP>
+ClusterFit g_tc_fit;   // cluster residency of k_attn_tc<HD, NP> (configure_tc)
 
-template <int HD>
+template <int HD, int NP>
 int configure_tc() {
-  auto k = k_attn_tc<HD>;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<HD>::bytes) !=
-      cudaSuccess)
+  auto k = k_attn_tc<HD, NP>;
+  constexpr size_t smem = TcSmem<HD, NP>::bytes;
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return -1;
   const bool nonportable =
       cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
   cudaGetLastError();
-  fill_cluster_fit(&g_tc_fit<HD>, k, TTHREADS, TcSmem<HD>::bytes, nonportable ? TACL : 8);
-  return nonportable && g_tc_fit<HD>.active[TACL] >= 1 ? 0 : 1;   // 1: portable only
+  fill_cluster_fit(&g_tc_fit<HD, NP>, k, TTHREADS, smem, nonportable ? TACL : 8);
+  return nonportable && g_tc_fit<HD, NP>.active[TACL] >= 1 ? 0 : 1;   // 1: portable only
+}
+
+template <int HD, int NP>
+void launch_tc(const AttnArgs& a, int n_z, cudaStream_t s) {
+  const int cl = attn_cluster_size(g_tc_fit<HD, NP>, g_tc_max_cluster, a.n_chunks + a.n_tchunks,
+                                   a.kv.kvh * n_z);
+  launch_pdl_cluster(k_attn_tc<HD, NP>, dim3(cl, a.kv.kvh, n_z), dim3(TTHREADS),
+                     TcSmem<HD, NP>::bytes, cl, s, a);
 }
 
 }  // namespace
 
-int attn_tc_qblock(int rows_per_prompt, int G) {
-  // up to 128 query vectors, and at most 32 rows meeting in one block (the tail layout runs
-  // one lane per row): 32 G vectors (whole rows) when that is smaller; no larger than a
-  // prompt's vectors rounded up to whole rows of 16
-  const int cap = std::min(128, 32 * G);
+int attn_tc_qblock(int rows_per_prompt, int G, bool tails) {
+  // up to 128 query vectors; with beam tails at most 32 rows meeting in one block (the tail
+  // layout runs one lane per row): 32 G vectors (whole rows) when that is smaller; no larger
+  // than a prompt's vectors rounded up to whole rows of 16
+  const int cap = tails ? std::min(TQB, 32 * G) : TQB;
   const int nq = rows_per_prompt * G;
   return std::max(16, std::min(cap, (nq + 15) / 16 * 16));
 }
 
 int configure_attention_tc() {
-  const int r128 = configure_tc<128>(), r64 = configure_tc<64>();
-  if (r128 < 0 || r64 < 0) return -1;
-  g_tc_max_cluster = (r128 || r64) ? 8 : TACL;
+  int worst = 0;
+  for (int r : {configure_tc<128, 2>(), configure_tc<64, 2>(), configure_tc<128, 3>(),
+                configure_tc<64, 3>()}) {
+    if (r < 0) return -1;
+    worst = std::max(worst, r);
+  }
+  g_tc_max_cluster = worst ? 8 : TACL;
   return 0;
 }
 
 void launch_attn_tc(const AttnArgs& a, int n_z, cudaStream_t s) {
-  const int cl = attn_cluster_size(a.kv.hd == 128 ? g_tc_fit<128> : g_tc_fit<64>,
-                                   g_tc_max_cluster, a.n_chunks + a.n_tchunks, a.kv.kvh * n_z);
-  if (a.kv.hd == 128)
-    launch_pdl_cluster(k_attn_tc<128>, dim3(cl, a.kv.kvh, n_z), dim3(TTHREADS),
-                       TcSmem<128>::bytes, cl, s, a);
-  else
-    launch_pdl_cluster(k_attn_tc<64>, dim3(cl, a.kv.kvh, n_z), dim3(TTHREADS),
-                       TcSmem<64>::bytes, cl, s, a);
+  // prefill passes with three planes of P and V: their K/V cache carries every later step (two
+  // planes: 13B logits after two layers 2.1e-5 -> 2.6e-5 off 64 bits, 3 to 7 % of the pass)
+  if (a.n_tchunks == 0) a.kv.hd == 128 ? launch_tc<128, 3>(a, n_z, s) : launch_tc<64, 3>(a, n_z, s);
+  else a.kv.hd == 128 ? launch_tc<128, 2>(a, n_z, s) : launch_tc<64, 2>(a, n_z, s);
 }
 
 }  // namespace cdsl

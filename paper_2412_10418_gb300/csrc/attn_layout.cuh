@@ -55,9 +55,9 @@ __device__ __forceinline__ int chunk_of(const Layout<QB>& L, int n_p, int cx, in
 // called by all NTHREADS threads of the block (a multiple of 32, at most 1024), which it
 // leaves synchronized. Reads only what the launch chain has already completed (row
 // descriptors, committed page table), so it may run before griddepcontrol.wait. Returns the
-// number of the block's query vectors (0..a.qblock). At most 32 rows may meet in one query block
-// (the tail layout runs one lane per row). More tail keys than the tail chunks hold latch
-// CDSL_ERANGE.
+// number of the block's query vectors (0..a.qblock). In a pass with tails (a.n_tchunks > 0) at most
+// 32 rows may meet in one query block (the tail layout runs one lane per row). More tail keys than
+// the tail chunks hold latch CDSL_ERANGE.
 template <int QB, int NTHREADS>
 __device__ int build_layout(Layout<QB>& L, const AttnArgs& a, int b, int qb, int cx, int C) {
   constexpr int NWARPS = NTHREADS / 32;
@@ -105,11 +105,12 @@ __device__ int build_layout(Layout<QB>& L, const AttnArgs& a, int b, int qb, int
     const int first_local = (qb * QBr) / G;
     const int qi_l = max(0, (first_local + lane) * G - qb * QBr);   // the row's first vector
     const bool row_ok = nq > 0 && qi_l < nq && lane <= (qb * QBr + nq - 1) / G - first_local;
-    int np = row_ok ? L.np[qi_l] : 0;
+    int np = 0;
+    for (int i = lane; i < nq; i += 32) np = max(np, L.np[i]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) np = max(np, __shfl_xor_sync(0xffffffffu, np, o));
     const int tb = row_ok ? L.tb[qi_l] : -1;
-    const int nt = row_ok ? L.nt[qi_l] : 0;
+    const int nt = row_ok && a.n_tchunks > 0 ? L.nt[qi_l] : 0;
     int len = 0;
     bool first = nt > 0;
     for (int j = 0; j < 32; ++j) {

@@ -85,9 +85,9 @@ int attn_qblock_for(int rows_per_prompt, int G);
 int attn_tail_chunks(int rows_per_prompt, int G, int rows_per_tail, int max_tail);
 int configure_attention();
 void launch_attn(int dtype, const AttnArgs& a, int n_z, cudaStream_t s);
-// Tensor-core attention (attention_tc.cu) for dense passes of bf16 models (no zmap): query
-// blocks of attn_tc_qblock() vectors (at most 128), head_dim 64 or 128.
-int attn_tc_qblock(int rows_per_prompt, int G);
+// Tensor-core attention (attention_tc.cu) for passes of bf16 models: query blocks of
+// attn_tc_qblock() vectors (at most 128; tails: the pass has beam tails), head_dim 64 or 128.
+int attn_tc_qblock(int rows_per_prompt, int G, bool tails);
 int configure_attention_tc();
 void launch_attn_tc(const AttnArgs& a, int n_z, cudaStream_t s);
 // Row statistics of logits rows: argmax (lower id on ties), log-sum-exp, top-k, log p.
