@@ -487,8 +487,6 @@ bool use_attn_tc(const cdsl_ctx* c, int rows_per_prompt, int G) {
   return c->dtype == CDSL_DTYPE_BF16 && rows_per_prompt * G >= kAttnTcMinVectors;
 }
 
-// One forward pass of a model over R rows described by `rows`; for lm_rows > 0 the final
-// norm + LM head run over rows gather[i] (or the first lm_rows rows) into logits.
 // Attention layout of a pass: rows per prompt (dense z mapping) or a host-built z map.
 struct AttnPass {
   int rows_per_prompt = 0;            // dense: z = b * qb_count + qb; prefill: of the prompt
@@ -499,12 +497,12 @@ struct AttnPass {
   int n_tchunks = 0;                  // tail-key chunks (attn_tail_chunks)
 };
 
-// One forward pass of a model over R rows described by `rows`; for lm_rows > 0 the final
+// One forward pass of a model over R rows, planned into `rows` by `plan`; for lm_rows > 0 the final
 // norm + LM head run over rows gather[i] (or the first lm_rows rows) into logits. RMSNorm is
 // folded into the GEMMs (the residual epilogues write h . g_next and the partial sums of h^2,
 // the consumers scale by the row factor); only a gathered LM input is normalized by a kernel.
 // With want_head, the last layer also leaves the reward-head partials in c->ss_hw.
-void forward(cdsl_ctx* c, ModelW& m, const RowDesc* rows, int R, int lm_rows,
+void forward(cdsl_ctx* c, ModelW& m, const RowPlan& plan, RowDesc* rows, int R, int lm_rows,
              const int32_t* gather, float* logits, bool want_head, const AttnPass& ap) {
   const cdsl_model_cfg& cfg = m.cfg;
   const int D = cfg.d_model, hd = cfg.head_dim, H = cfg.n_heads, KVH = cfg.n_kv_heads;
@@ -540,7 +538,7 @@ void forward(cdsl_ctx* c, ModelW& m, const RowDesc* rows, int R, int lm_rows,
     if (head) { a.head_w = c->head_w; a.out_hw = c->ss_hw; }
   };
   timed(c, K_EMBED, 0, 0, [&] {
-    launch_embed(c->dtype, rows, R, m.embed, D, c->h, c->X1, c->act_plane,
+    launch_embed(c->dtype, plan, rows, R, m.embed, D, c->h, c->X1, c->act_plane,
                  m.layers[0][W_ATTN_NORM], c->ss_a, ld_ss, s);
   });
   for (int l = 0; l < L; ++l) {
@@ -557,6 +555,7 @@ void forward(cdsl_ctx* c, ModelW& m, const RowDesc* rows, int R, int lm_rows,
     normed_input(q, c->ss_a);
     gemm(c, q);
     at.layer = l;
+    at.rows_late = l == 0;   // (the embedding kernel plans them)
     timed(c, K_ATTN, 0, 0, [&] {
       at.stamp = c->cur_stamp;
       if (attn_tc) launch_attn_tc(at, n_z, s);
@@ -599,12 +598,11 @@ void forward(cdsl_ctx* c, ModelW& m, const RowDesc* rows, int R, int lm_rows,
 
 void do_lookahead(cdsl_ctx* c) {
   for (int j = 1; j <= c->d; ++j) {
-    timed(c, K_STEPLOGIC, 0, 0, [&] { launch_plan_draft(c->st, j, c->dft.spb, c->rows_d, c->stream); });
     const int R = c->B * c->k + (j == 1 ? c->B : 0);
     AttnPass ap;
     ap.rows_per_prompt = c->k + (j == 1 ? 1 : 0);
     ap.n_tchunks = attn_tail_chunks(ap.rows_per_prompt, group_size(c->dcfg), 1, j);
-    forward(c, c->dft, c->rows_d, R, c->B * c->k, nullptr, c->logits, false, ap);
+    forward(c, c->dft, RowPlan{c->st, PLAN_DRAFT, j, c->dft.spb}, c->rows_d, R, c->B * c->k, nullptr, c->logits, false, ap);
     RowStatsArgs a{};
     a.logits = c->logits; a.R = c->B * c->k; a.V = c->V; a.k = c->k;
     a.x_out = c->st.x; a.logq_out = c->st.logq; a.out_stride = c->d; a.out_off = j - 1;
@@ -617,11 +615,11 @@ void do_lookahead(cdsl_ctx* c) {
 }
 
 void do_verify(cdsl_ctx* c) {
-  timed(c, K_STEPLOGIC, 0, 0, [&] { launch_plan_verify(c->st, c->rows_v, c->stream); });
   AttnPass ap;
   ap.rows_per_prompt = c->k * (c->d + 1);
   ap.n_tchunks = attn_tail_chunks(ap.rows_per_prompt, group_size(c->tcfg), c->d + 1, c->d + 1);
-  forward(c, c->tgt, c->rows_v, c->R_v, c->R_v, nullptr, c->logits, c->run.reward_head != 0, ap);
+  forward(c, c->tgt, RowPlan{c->st, PLAN_VERIFY, 0, 0}, c->rows_v, c->R_v, c->R_v, nullptr,
+          c->logits, c->run.reward_head != 0, ap);
   RowStatsArgs a{};
   a.logits = c->logits; a.R = c->R_v; a.V = c->V; a.k = c->k; a.dp1 = c->d + 1;
   a.next_x = c->st.x; a.amax = c->st.v_amax; a.logp = c->st.v_logp; a.topk = c->st.v_topk;
@@ -643,11 +641,10 @@ void do_verify(cdsl_ctx* c) {
 void do_step1_round(cdsl_ctx* c) {
   const int B = c->B, d = c->d;
   for (int j = 1; j <= d; ++j) {
-    timed(c, K_STEPLOGIC, 0, 0, [&] { launch_plan_s1_draft(c->st, j, c->rows_d, c->stream); });
     AttnPass ap;
     ap.rows_per_prompt = j == 1 ? 2 : 1;
     ap.n_tchunks = s1_tail_chunks_d(c->dcfg, c->run, j);
-    forward(c, c->dft, c->rows_d, ap.rows_per_prompt * B, B, nullptr, c->logits, false, ap);
+    forward(c, c->dft, RowPlan{c->st, PLAN_S1_DRAFT, j, 0}, c->rows_d, ap.rows_per_prompt * B, B, nullptr, c->logits, false, ap);
     RowStatsArgs a{};
     a.logits = c->logits; a.R = B; a.V = c->V; a.k = c->k;
     a.x_out = c->st.s1_tok; a.logq_out = c->st.s1_logq; a.out_stride = d + 1; a.out_off = j;
@@ -657,11 +654,11 @@ void do_step1_round(cdsl_ctx* c) {
       launch_row_stats(a, c->stream);
     });
   }
-  timed(c, K_STEPLOGIC, 0, 0, [&] { launch_plan_s1_verify(c->st, c->rows_v, c->stream); });
   AttnPass ap;
   ap.rows_per_prompt = d + 2;
   ap.n_tchunks = s1_tail_chunks_t(c->tcfg, c->run);
-  forward(c, c->tgt, c->rows_v, c->R_s1, B, nullptr, c->logits, c->run.reward_head != 0, ap);
+  forward(c, c->tgt, RowPlan{c->st, PLAN_S1_VERIFY, 0, 0}, c->rows_v, c->R_s1, B, nullptr,
+          c->logits, c->run.reward_head != 0, ap);
   RowStatsArgs a{};
   a.logits = c->logits; a.R = B; a.V = c->V; a.k = c->k;
   a.topk = c->st.s1_topk; a.status = c->st.status;
@@ -679,9 +676,7 @@ void do_select(cdsl_ctx* c) {
   timed(c, K_STEPLOGIC, 0, 0, [&] { launch_select(c->st, c->tgt.kv, c->dft.kv, 1, c->stream); });
   if (c->run.step1_budget >= 2) do_step1_round(c);
   timed(c, K_STEPLOGIC, 0, 0, [&] {
-    launch_commit_kv(c->st, c->tgt.kv, c->tgt.spb, 0, c->stream);
-    launch_commit_kv(c->st, c->dft.kv, c->dft.spb, 1, c->stream);
-    launch_advance(c->st, c->stream);
+    launch_commit_kv(c->st, c->tgt.kv, c->dft.kv, c->tgt.spb, c->dft.spb, c->stream);
   });
 }
 
@@ -691,12 +686,20 @@ void copy_out(cdsl_ctx* c, void* dst, const void* src, size_t bytes) {
 
 void copy_select_outputs(cdsl_ctx* c, int32_t* beam, int32_t* state, int32_t* emitted,
                          int32_t* n_emitted, float* reward) {
-  const size_t B = c->B;
-  copy_out(c, beam, c->st.beam, B * 4);
-  copy_out(c, state, c->st.state, B * 4);
-  copy_out(c, emitted, c->st.emitted, B * (c->d + 1) * 4);
-  copy_out(c, n_emitted, c->st.n_emit, B * 4);
-  copy_out(c, reward, c->st.reward, B * c->k * 2 * 4);
+  const int B = c->B;
+  CopyOut o{};
+  int q = 0;
+  auto want = [&](void* dst, const void* src, int words) {
+    o.dst[q] = static_cast<uint32_t*>(dst);
+    o.src[q] = static_cast<const uint32_t*>(src);
+    o.n[q++] = dst ? words : 0;
+  };
+  want(beam, c->st.beam, B);
+  want(state, c->st.state, B);
+  want(emitted, c->st.emitted, B * (c->d + 1));
+  want(n_emitted, c->st.n_emit, B);
+  want(reward, c->st.reward, B * c->k * 2);
+  launch_copy_out(o, c->stream);
 }
 
 int bind_model(ModelW& m, const cdsl_model_cfg& cfg, const void* const* w, const char* name,
@@ -895,14 +898,14 @@ int32_t cdsl_prefill(cdsl_ctx* c, const int32_t* d_prompts, const int32_t* h_pro
     apt.zmap = &zt;
     apd.zmap = &zd;
     apt.n_chunks = apd.n_chunks = (maxpos + attn_chunk()) / attn_chunk();
-    forward(c, c->tgt, c->rows_p, R, nlm, c->lm_gather, c->logits, false, apt);
+    forward(c, c->tgt, RowPlan{}, c->rows_p, R, nlm, c->lm_gather, c->logits, false, apt);
     if (nlm) {
       RowStatsArgs a{};
       a.logits = c->logits; a.R = nlm; a.V = c->V; a.k = c->k;
       a.topk = st.roots; a.dst = c->lm_dst; a.status = st.status;
       launch_row_stats(a, s);
     }
-    forward(c, c->dft, c->rows_p, R, 0, nullptr, nullptr, false, apd);
+    forward(c, c->dft, RowPlan{}, c->rows_p, R, 0, nullptr, nullptr, false, apd);
     cudaStreamSynchronize(s);  // host row buffers are reused by the next chunk
     rows.clear(); gather.clear(); dst.clear();
   };

@@ -78,9 +78,11 @@ __global__ void __launch_bounds__(ATHREADS, 2) k_attn(AttnArgs a) {
   const int G = a.G, H = a.n_heads;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  // ---- this cluster's query vectors and this block's key slots. The rows (plan kernel), the
+  // ---- this cluster's query vectors and this block's key slots. The rows (embedding kernel), the
   //      committed page table and the tail layout come from kernels the launch chain has
-  //      already completed, so all of it precedes the wait.
+  //      already completed, so all of it precedes the wait -- except in layer 0, whose
+  //      embedding kernel may still be running.
+  if (a.rows_late) pdl_wait();
   const int nq = attn::build_layout<QB, ATHREADS>(L, a, b, qb, cx, C);
   const int nb_chunks = L.nb;                     // chunk_of(L, n_p, cx, C, 0 .. nb_chunks - 1)
   const int maxnp = L.maxnp;

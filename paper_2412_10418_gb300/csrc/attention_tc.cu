@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
   const int warp = threadIdx.x >> 5;
 
   // ---- query vectors and key slots (before the wait: inputs of completed kernels only)
+  if (a.rows_late) pdl_wait();
   const int nq = attn::build_layout<TQB, TTHREADS>(L, a, b, qb, cx, C);
   const int nb_chunks = L.nb;                     // chunk_of(L, n_p, cx, C, 0 .. nb_chunks - 1)
   if (a.stamp) attn::count_bytes<TQB, TTHREADS, HD>(L, stamp, qb, cx, nb_chunks, nq, &s_nkeys);

@@ -3,6 +3,8 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "gemm.cuh"
 #include "kernels.h"
 
@@ -38,16 +40,161 @@ __device__ unsigned long long block_max_u64(unsigned long long v, unsigned long 
   return red[0];
 }
 
+// ------------------------------------------------------------------------------ plans
+// Row descriptors of the passes of a step, from the device-resident state. The embedding kernel
+// computes its row's descriptor and leaves it for the pass's other kernels: a launch of its own
+// for them cost about 2.5 us per pass.
+
+// Draft call j (1..d): beam rows (b, i) carry c_bi (j = 1) or x_bi,j-1 at position L + j - 1,
+// see the prefix and their own tail slots 0..j-1. Call 1 adds one row per prompt: the pending
+// token L-1 of a fully accepted step, written straight into the draft prefix pages.
+__device__ RowDesc plan_draft(const StepState& st, int j, int spb, int r) {
+  const int nbk = st.B * st.k;
+  RowDesc rd;
+  if (r < nbk) {
+    const int b = r / st.k;
+    const int L = st.len[b];
+    rd.b = b;
+    rd.pos = L + j - 1;
+    rd.token = (j == 1) ? st.roots[r] : st.x[r * st.d + j - 2];
+    rd.n_prefix = L;
+    rd.tail_base = r * spb;
+    rd.n_tail = j;
+    rd.kv_dst = r * spb + j - 1;
+    rd.out_idx = r;
+  } else {
+    const int b = r - nbk;
+    const int L = st.len[b];
+    rd.b = b;
+    rd.tail_base = 0;
+    rd.n_tail = 0;
+    rd.out_idx = -1;
+    if (st.pend[b]) {
+      rd.pos = L - 1;
+      rd.token = st.tokens[b * st.lcap + L - 1];
+      rd.n_prefix = L;
+      rd.kv_dst = KV_PREFIX;
+    } else {  // idle row: reads position 0, stores nothing
+      rd.pos = 0;
+      rd.token = 0;
+      rd.n_prefix = 1;
+      rd.kv_dst = KV_NONE;
+    }
+  }
+  return rd;
+}
+
+// Verify rows (b, i, j), j = 0..d: token c_bi (j = 0) or x_bi,j at position L + j; they see
+// the prefix and their beam's tail slots 0..j (causal within the beam, nothing across beams).
+__device__ RowDesc plan_verify(const StepState& st, int r) {
+  const int dp1 = st.d + 1;
+  const int bi = r / dp1, j = r % dp1, b = bi / st.k;
+  const int L = st.len[b];
+  RowDesc rd;
+  rd.b = b;
+  rd.pos = L + j;
+  rd.token = (j == 0) ? st.roots[bi] : st.x[bi * st.d + j - 1];
+  rd.n_prefix = L;
+  rd.tail_base = bi * dp1;
+  rd.n_tail = j + 1;
+  rd.kv_dst = r;
+  rd.out_idx = r;
+  return rd;
+}
+
+// Step-1 round 2, draft call j (1..d), in the round's own tail region of d+1 slots per prompt
+// (slot 0 c_1, slot 1 x', slot j lh_j-1): rows [0, B) carry x' at L + 1 (j = 1, which also
+// records x' = argmax M_p(pfx + c_1), verify row (b, 1, 0)) or lh_j-1 at L + j; rows [B, 2B)
+// of call 1 carry c_1 at L.
+__device__ RowDesc plan_s1_draft(const StepState& st, int j, int r) {
+  const int B = st.B, dp1 = st.d + 1;
+  const int b = r % B;
+  const int L = st.len[b], base = st.s1_dbase + b * dp1;
+  RowDesc rd;
+  rd.b = b;
+  rd.n_prefix = L;
+  rd.tail_base = base;
+  if (r >= B) {
+    rd.pos = L;
+    rd.token = st.roots[b * st.k];
+    rd.n_tail = 1;
+    rd.kv_dst = base;
+    rd.out_idx = -1;
+  } else if (j == 1) {
+    const int xp = st.v_amax[b * st.k * dp1];
+    st.s1_tok[b * dp1] = xp;
+    rd.pos = L + 1;
+    rd.token = xp;
+    rd.n_tail = 2;
+    rd.kv_dst = base + 1;
+    rd.out_idx = b;
+  } else {
+    rd.pos = L + j;
+    rd.token = st.s1_tok[b * dp1 + j - 1];
+    rd.n_tail = j + 1;
+    rd.kv_dst = base + j;
+    rd.out_idx = b;
+  }
+  return rd;
+}
+
+// Step-1 round 2, the target pass, in its tail region of d+2 slots per prompt (c_1, x',
+// lh_1..lh_d): rows [0, B) x' at L + 1 (the LM rows: M_p(pfx + c_1 + x')), [B, 2B) c_1 at L,
+// then lh_j at L + 1 + j, prompt-major (the reward head reads lh_d's row).
+__device__ RowDesc plan_s1_verify(const StepState& st, int r) {
+  const int B = st.B, d = st.d, dp1 = d + 1;
+  int b, slot;
+  if (r < B) {
+    b = r; slot = 1;
+  } else if (r < 2 * B) {
+    b = r - B; slot = 0;
+  } else {
+    b = (r - 2 * B) / d; slot = 2 + (r - 2 * B) % d;
+  }
+  const int L = st.len[b], base = st.s1_tbase + b * (d + 2);
+  RowDesc rd;
+  rd.b = b;
+  rd.pos = L + slot;
+  rd.token = slot == 0 ? st.roots[b * st.k] : st.s1_tok[b * dp1 + slot - 1];
+  rd.n_prefix = L;
+  rd.tail_base = base;
+  rd.n_tail = slot + 1;
+  rd.kv_dst = base + slot;
+  rd.out_idx = r < B ? b : -1;
+  return rd;
+}
+
+__device__ RowDesc plan_row(const RowPlan& p, int r) {
+  switch (p.kind) {
+    case PLAN_DRAFT: return plan_draft(p.st, p.j, p.spb, r);
+    case PLAN_VERIFY: return plan_verify(p.st, r);
+    case PLAN_S1_DRAFT: return plan_s1_draft(p.st, p.j, r);
+    default: return plan_s1_verify(p.st, r);
+  }
+}
+
 // ------------------------------------------------------------------------------ embedding
-// h = E[token]; also the first GEMM input x = h . g (GEMM-input format) and the 32-feature
-// partial sums of h^2 from which the consuming GEMM takes the RMSNorm row scale.
+// One block per row: its descriptor (planned here, or read where the host built the rows: prefill),
+// h = E[token], the first GEMM input x = h . g (GEMM-input format) and the 32-feature partial
+// sums of h^2 from which the consuming GEMM takes the RMSNorm row scale.
 template <typename T>
-__global__ void k_embed(const RowDesc* rows, const T* E, int D, float* h, T* x, size_t plane,
-                        const T* g, float* ss, int ld_ss) {
+__global__ void k_embed(const RowPlan p, RowDesc* rows, const T* E, int D, float* h, T* x,
+                        size_t plane, const T* g, float* ss, int ld_ss) {
   pdl_wait();
   pdl_launch_dependents();
+  __shared__ int s_token;
   const int r = blockIdx.x;
-  const T* e = E + (size_t)rows[r].token * D;
+  if (threadIdx.x == 0) {
+    if (p.kind == PLAN_HOST) {
+      s_token = rows[r].token;
+    } else {
+      const RowDesc rd = plan_row(p, r);
+      rows[r] = rd;
+      s_token = rd.token;
+    }
+  }
+  __syncthreads();
+  const T* e = E + (size_t)s_token * D;
   for (int c0 = 0; c0 < D; c0 += blockDim.x) {   // blockDim is a multiple of 32, D of 64
     const int c = c0 + threadIdx.x;
     const float v = c < D ? to_f32<T>(e[c]) : 0.f;
@@ -207,143 +354,6 @@ __global__ void __launch_bounds__(RS_THREADS) k_row_stats(RowStatsArgs a) {
   }
 }
 
-// ------------------------------------------------------------------------------ plans
-// Draft call j (1..d): beam rows (b, i) carry c_bi (j = 1) or x_bi,j-1 at position L + j - 1,
-// see the prefix and their own tail slots 0..j-1. Call 1 adds one row per prompt: the pending
-// token L-1 of a fully accepted step, written straight into the draft prefix pages.
-__global__ void k_plan_draft(StepState st, int j, int spb, RowDesc* rows) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nbk = st.B * st.k;
-  if (r < nbk) {
-    const int b = r / st.k;
-    const int L = st.len[b];
-    RowDesc rd;
-    rd.b = b;
-    rd.pos = L + j - 1;
-    rd.token = (j == 1) ? st.roots[r] : st.x[r * st.d + j - 2];
-    rd.n_prefix = L;
-    rd.tail_base = r * spb;
-    rd.n_tail = j;
-    rd.kv_dst = r * spb + j - 1;
-    rd.out_idx = r;
-    rows[r] = rd;
-  } else if (j == 1 && r < nbk + st.B) {
-    const int b = r - nbk;
-    const int L = st.len[b];
-    RowDesc rd;
-    rd.b = b;
-    rd.tail_base = 0;
-    rd.n_tail = 0;
-    rd.out_idx = -1;
-    if (st.pend[b]) {
-      rd.pos = L - 1;
-      rd.token = st.tokens[b * st.lcap + L - 1];
-      rd.n_prefix = L;
-      rd.kv_dst = KV_PREFIX;
-    } else {  // idle row: reads position 0, stores nothing
-      rd.pos = 0;
-      rd.token = 0;
-      rd.n_prefix = 1;
-      rd.kv_dst = KV_NONE;
-    }
-    rows[r] = rd;
-  }
-}
-
-// Verify rows (b, i, j), j = 0..d: token c_bi (j = 0) or x_bi,j at position L + j; they see
-// the prefix and their beam's tail slots 0..j (causal within the beam, nothing across beams).
-__global__ void k_plan_verify(StepState st, RowDesc* rows) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int dp1 = st.d + 1;
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= st.B * st.k * dp1) return;
-  const int bi = r / dp1, j = r % dp1, b = bi / st.k;
-  const int L = st.len[b];
-  RowDesc rd;
-  rd.b = b;
-  rd.pos = L + j;
-  rd.token = (j == 0) ? st.roots[bi] : st.x[bi * st.d + j - 1];
-  rd.n_prefix = L;
-  rd.tail_base = bi * dp1;
-  rd.n_tail = j + 1;
-  rd.kv_dst = r;
-  rd.out_idx = r;
-  rows[r] = rd;
-}
-
-// Step-1 round 2, draft call j (1..d), in the round's own tail region of d+1 slots per prompt
-// (slot 0 c_1, slot 1 x', slot j lh_j-1): rows [0, B) carry x' at L + 1 (j = 1, which also
-// records x' = argmax M_p(pfx + c_1), verify row (b, 1, 0)) or lh_j-1 at L + j; rows [B, 2B)
-// of call 1 carry c_1 at L.
-__global__ void k_plan_s1_draft(StepState st, int j, RowDesc* rows) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int B = st.B, dp1 = st.d + 1;
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= (j == 1 ? 2 * B : B)) return;
-  const int b = r % B;
-  const int L = st.len[b], base = st.s1_dbase + b * dp1;
-  RowDesc rd;
-  rd.b = b;
-  rd.n_prefix = L;
-  rd.tail_base = base;
-  if (r >= B) {
-    rd.pos = L;
-    rd.token = st.roots[b * st.k];
-    rd.n_tail = 1;
-    rd.kv_dst = base;
-    rd.out_idx = -1;
-  } else if (j == 1) {
-    const int xp = st.v_amax[b * st.k * dp1];
-    st.s1_tok[b * dp1] = xp;
-    rd.pos = L + 1;
-    rd.token = xp;
-    rd.n_tail = 2;
-    rd.kv_dst = base + 1;
-    rd.out_idx = b;
-  } else {
-    rd.pos = L + j;
-    rd.token = st.s1_tok[b * dp1 + j - 1];
-    rd.n_tail = j + 1;
-    rd.kv_dst = base + j;
-    rd.out_idx = b;
-  }
-  rows[r] = rd;
-}
-
-// Step-1 round 2, the target pass, in its tail region of d+2 slots per prompt (c_1, x',
-// lh_1..lh_d): rows [0, B) x' at L + 1 (the LM rows: M_p(pfx + c_1 + x')), [B, 2B) c_1 at L,
-// then lh_j at L + 1 + j, prompt-major (the reward head reads lh_d's row).
-__global__ void k_plan_s1_verify(StepState st, RowDesc* rows) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int B = st.B, d = st.d, dp1 = d + 1;
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= B * (d + 2)) return;
-  int b, slot;
-  if (r < B) {
-    b = r; slot = 1;
-  } else if (r < 2 * B) {
-    b = r - B; slot = 0;
-  } else {
-    b = (r - 2 * B) / d; slot = 2 + (r - 2 * B) % d;
-  }
-  const int L = st.len[b], base = st.s1_tbase + b * (d + 2);
-  RowDesc rd;
-  rd.b = b;
-  rd.pos = L + slot;
-  rd.token = slot == 0 ? st.roots[b * st.k] : st.s1_tok[b * dp1 + slot - 1];
-  rd.n_prefix = L;
-  rd.tail_base = base;
-  rd.n_tail = slot + 1;
-  rd.kv_dst = base + slot;
-  rd.out_idx = r < B ? b : -1;
-  rows[r] = rd;
-}
-
 // ------------------------------------------------------------------------------ decision
 __device__ void alloc_pages(const KvStore& kv, int b, int from, int to, int32_t* next_page,
                             int32_t* status) {
@@ -359,7 +369,6 @@ __device__ void alloc_pages(const KvStore& kv, int b, int from, int to, int32_t*
   }
 }
 
-// One warp per prompt, one lane per beam: n_b, rewards, b*, state, emission, page allocation.
 // Draw number c of the SplitMix64 generator seeded with `seed` (Steele, Lea, Flood, 2014:
 // state_c = seed + (c + 1) * golden gamma, output = the variant-13 mix of the state), reduced
 // to its top 24 bits as a float in [0, 1) (exact in float32).
@@ -371,6 +380,41 @@ __device__ __forceinline__ float uniform24(uint32_t seed, unsigned long long c) 
   return (float)(z >> 40) * (1.0f / 16777216.0f);
 }
 
+// pfx <- pfx + O, T <- T + O; the next beams are the top-k of the winner's row cnt-1 (after a
+// Step-1 round-2 emission: of M_p(pfx + c_1 + x')). The warp of prompt b, whose emission the
+// caller has written; k_commit_kv then copies the K/V rows behind the new length.
+__device__ void advance(const StepState& st, int b, int lane) {
+  __syncwarp();
+  const int k = st.k, d = st.d, dp1 = d + 1;
+  const int cnt = st.n_emit[b];
+  if (cnt <= 0) return;
+  const int L = st.len[b], bs = st.beam[b];
+  if (lane < cnt) st.tokens[b * st.lcap + L + lane] = st.emitted[b * dp1 + lane];
+  uint32_t bits = 0;
+  if (lane < st.nk) {
+    const int kwq = st.kw[b * st.nk + lane];
+    for (int t = 0; t < cnt; ++t)
+      if (st.emitted[b * dp1 + t] == kwq) bits = 1u << lane;
+  }
+  for (int o = 16; o > 0; o >>= 1) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
+  const bool s1 = st.s1_used[b] != 0;
+  const int root_row = (b * k + bs) * dp1 + cnt - 1;
+  if (lane < k)
+    st.roots[b * k + lane] = s1 ? st.s1_topk[b * k + lane] : st.v_topk[root_row * k + lane];
+  __syncwarp();   // every lane has read the old length
+  if (lane == 0) {
+    st.cov[b] |= bits;
+    st.len[b] = L + cnt;
+    st.gen[b] += cnt;
+    st.pend[b] = (!s1 && cnt == dp1) ? 1 : 0;
+    atomicAdd((unsigned long long*)&st.counters[3], (unsigned long long)cnt);
+    if (st.state[b] == 1) atomicAdd((unsigned long long*)&st.counters[4], 1ull);
+    atomicAdd((unsigned long long*)&st.counters[5], 1ull);
+  }
+}
+
+// One warp per prompt, one lane per beam: n_b, rewards, b*, state, emission; with commit also page
+// allocation and (Step-1 budget below 2) the advance.
 __global__ void k_select(StepState st, KvStore tkv, KvStore dkv, int commit) {
   pdl_wait();
   pdl_launch_dependents();
@@ -457,23 +501,22 @@ __global__ void k_select(StepState st, KvStore tkv, KvStore dkv, int commit) {
     // budget 2: round 1 failed in S2/S3, round 2 may still replace this Step-2 emission
     st.s1_need[b] = (!s1 && nb < st.n_min && st.step1 >= 2 && !(rf1 >= st.r_t)) ? 1 : 0;
     st.s1_used[b] = 0;
-    if (!commit) return;
-    const int L = st.len[b];
-    alloc_pages(tkv, b, L, L + cnt, st.next_page + 0, st.status);
-    alloc_pages(dkv, b, L, L + cnt, st.next_page + 1, st.status);
+    if (commit) {
+      const int L = st.len[b];
+      alloc_pages(tkv, b, L, L + cnt, st.next_page + 0, st.status);
+      alloc_pages(dkv, b, L, L + cnt, st.next_page + 1, st.status);
+    }
   }
+  if (commit && st.step1 < 2) advance(st, b, lane);   // budget 2: k_select_s1 does
 }
 
 // Step-1 round 2 (Alg. 1 S2/S3, Sec. 3.2.3, budget b = 2): X = [c_1, x'] with the lookahead
 // lh of x'; R(T + X + lh) from the keyword bits and M_p's hidden state at lh_d (the same
-// arithmetic as the verify rows' head). One warp per prompt.
-__global__ void k_select_s1(StepState st, KvStore tkv, KvStore dkv, const float* ss,
-                            const float* hw, int norm_D, int ld_ss, float eps) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int b = blockIdx.x, lane = threadIdx.x;
+// arithmetic as the verify rows' head). The warp of prompt b.
+__device__ void s1_decide(const StepState& st, const KvStore& tkv, const KvStore& dkv,
+                          const float* ss, const float* hw, int norm_D, int ld_ss, float eps, int b,
+                          int lane) {
   const int d = st.d, dp1 = d + 1;
-  if (!st.s1_need[b]) return;
   const int c1 = st.roots[b * st.k];
   uint32_t bits = 0;
   if (lane < st.nk) {
@@ -509,17 +552,38 @@ __global__ void k_select_s1(StepState st, KvStore tkv, KvStore dkv, const float*
   }
 }
 
-// Copy the winner's tail K/V rows 0..cnt-1 to prefix positions L..L+cnt-1 (after a Step-1
-// round-2 emission: rows 0, 1 of the round's tail region).
-__global__ void k_commit_kv(StepState st, KvStore kv, int spb, int is_draft) {
+// Step-1 round 2's decision where round 1 failed, then the advance of every prompt (one warp each).
+__global__ void k_select_s1(StepState st, KvStore tkv, KvStore dkv, const float* ss,
+                            const float* hw, int norm_D, int ld_ss, float eps) {
   pdl_wait();
   pdl_launch_dependents();
-  const int b = blockIdx.x, layer = blockIdx.y, kvsel = blockIdx.z;
+  const int b = blockIdx.x, lane = threadIdx.x;
+  if (st.s1_need[b]) s1_decide(st, tkv, dkv, ss, hw, norm_D, ld_ss, eps, b, lane);
+  advance(st, b, lane);
+}
+
+// Copy the winner's tail K/V rows 0..cnt-1 to prefix positions L..L+cnt-1 of both models (after a
+// Step-1 round-2 emission: rows 0, 1 of the round's tail region); L is the length before the
+// advance. blockIdx.z: K and V of the target, then of the draft.
+__global__ void k_commit_kv(StepState st, KvStore tkv, KvStore dkv, int t_spb, int d_spb) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int b = blockIdx.x, layer = blockIdx.y, kvsel = blockIdx.z & 1;
+  const bool is_draft = blockIdx.z >= 2;
+  const KvStore& kv = is_draft ? dkv : tkv;
+  const int spb = is_draft ? d_spb : t_spb;
+  if (b == 0 && layer == 0 && blockIdx.z == 0 && threadIdx.x == 0) {
+    const int rounds = st.step1 >= 2 ? 2 : 1;   // the Step-1 round runs every step
+    st.counters[0] += 1;                        // steps
+    st.counters[1] += st.d * rounds;            // draft forward passes
+    st.counters[2] += rounds;                   // target forward passes
+  }
+  if (layer >= kv.n_layers) return;
   int cnt = st.n_emit[b];
-  const bool s1 = st.s1_used[b] != 0;
-  if (is_draft && !s1) cnt = min(cnt, st.d);
   if (cnt <= 0) return;
-  const int bs = st.beam[b], L = st.len[b];
+  const bool s1 = st.s1_used[b] != 0;
+  const int bs = st.beam[b], L = st.len[b] - cnt;
+  if (is_draft && !s1) cnt = min(cnt, st.d);
   const int src0 = !s1 ? (b * st.k + bs) * spb
                        : (is_draft ? st.s1_dbase + b * (st.d + 1) : st.s1_tbase + b * (st.d + 2));
   const int per_row = kv.kvh * kv.hd;
@@ -534,42 +598,14 @@ __global__ void k_commit_kv(StepState st, KvStore kv, int spb, int is_draft) {
   }
 }
 
-// pfx <- pfx + O, T <- T + O; the next beams are the top-k of the winner's row cnt-1.
-__global__ void k_advance(StepState st) {
+// The outputs of a decision to the caller's buffers: words of each that is wanted.
+__global__ void k_copy_out(const CopyOut c) {
   pdl_wait();
   pdl_launch_dependents();
-  const int b = blockIdx.x, lane = threadIdx.x;
-  const int k = st.k, d = st.d, dp1 = d + 1;
-  if (b == 0 && lane == 0) {
-    const int rounds = st.step1 >= 2 ? 2 : 1;   // the Step-1 round runs every step
-    st.counters[0] += 1;                        // steps
-    st.counters[1] += d * rounds;               // draft forward passes
-    st.counters[2] += rounds;                   // target forward passes
-  }
-  const int cnt = st.n_emit[b];
-  if (cnt <= 0) return;
-  const int L = st.len[b], bs = st.beam[b];
-  if (lane < cnt) st.tokens[b * st.lcap + L + lane] = st.emitted[b * dp1 + lane];
-  uint32_t bits = 0;
-  if (lane < st.nk) {
-    const int kwq = st.kw[b * st.nk + lane];
-    for (int t = 0; t < cnt; ++t)
-      if (st.emitted[b * dp1 + t] == kwq) bits = 1u << lane;
-  }
-  for (int o = 16; o > 0; o >>= 1) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
-  const bool s1 = st.s1_used[b] != 0;   // next roots: top-k of M_p(pfx + c_1 + x')
-  const int root_row = (b * k + bs) * dp1 + cnt - 1;
-  if (lane < k)
-    st.roots[b * k + lane] = s1 ? st.s1_topk[b * k + lane] : st.v_topk[root_row * k + lane];
-  if (lane == 0) {
-    st.cov[b] |= bits;
-    st.len[b] = L + cnt;
-    st.gen[b] += cnt;
-    st.pend[b] = (!s1 && cnt == dp1) ? 1 : 0;
-    atomicAdd((unsigned long long*)&st.counters[3], (unsigned long long)cnt);
-    if (st.state[b] == 1) atomicAdd((unsigned long long*)&st.counters[4], 1ull);
-    atomicAdd((unsigned long long*)&st.counters[5], 1ull);
-  }
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+#pragma unroll
+  for (int q = 0; q < CopyOut::N; ++q)
+    if (i < c.n[q]) c.dst[q][i] = c.src[q][i];
 }
 
 __global__ void k_rope_table(float2* table, int n_pos, int hd, double theta) {
@@ -597,9 +633,10 @@ __global__ void k_rope_table(float2* table, int n_pos, int hd, double theta) {
     }                                                          \
   } while (0)
 
-void launch_embed(int dtype, const RowDesc* rows, int R, const void* embed, int D, float* h,
-                  void* x, size_t plane, const void* g, float* ss, int ld_ss, cudaStream_t s) {
-  DISPATCH(dtype, launch_pdl(k_embed<T>, dim3(R), dim3(256), 0, s, rows, (const T*)embed, D, h,
+void launch_embed(int dtype, const RowPlan& p, RowDesc* rows, int R, const void* embed, int D,
+                  float* h, void* x, size_t plane, const void* g, float* ss, int ld_ss,
+                  cudaStream_t s) {
+  DISPATCH(dtype, launch_pdl(k_embed<T>, dim3(R), dim3(256), 0, s, p, rows, (const T*)embed, D, h,
                              (T*)x, plane, (const T*)g, ss, ld_ss));
 }
 
@@ -614,26 +651,6 @@ void launch_row_stats(const RowStatsArgs& a, cudaStream_t s) {
   launch_pdl(k_row_stats, dim3(a.R), dim3(RS_THREADS), 0, s, a);
 }
 
-void launch_plan_draft(const StepState& st, int j, int spb, RowDesc* rows, cudaStream_t s) {
-  const int n = st.B * st.k + (j == 1 ? st.B : 0);
-  launch_pdl(k_plan_draft, dim3((n + 127) / 128), dim3(128), 0, s, st, j, spb, rows);
-}
-
-void launch_plan_verify(const StepState& st, RowDesc* rows, cudaStream_t s) {
-  const int n = st.B * st.k * (st.d + 1);
-  launch_pdl(k_plan_verify, dim3((n + 127) / 128), dim3(128), 0, s, st, rows);
-}
-
-void launch_plan_s1_draft(const StepState& st, int j, RowDesc* rows, cudaStream_t s) {
-  const int n = j == 1 ? 2 * st.B : st.B;
-  launch_pdl(k_plan_s1_draft, dim3((n + 127) / 128), dim3(128), 0, s, st, j, rows);
-}
-
-void launch_plan_s1_verify(const StepState& st, RowDesc* rows, cudaStream_t s) {
-  const int n = st.B * (st.d + 2);
-  launch_pdl(k_plan_s1_verify, dim3((n + 127) / 128), dim3(128), 0, s, st, rows);
-}
-
 void launch_select_s1(const StepState& st, KvStore tkv, KvStore dkv, const float* ss,
                       const float* hw, int norm_D, int ld_ss, float norm_eps, cudaStream_t s) {
   launch_pdl(k_select_s1, dim3(st.B), dim3(32), 0, s, st, tkv, dkv, ss, hw, norm_D, ld_ss,
@@ -644,13 +661,16 @@ void launch_select(const StepState& st, KvStore tkv, KvStore dkv, int commit, cu
   launch_pdl(k_select, dim3(st.B), dim3(32), 0, s, st, tkv, dkv, commit);
 }
 
-void launch_commit_kv(const StepState& st, KvStore kv, int spb, int is_draft, cudaStream_t s) {
-  dim3 grid(st.B, kv.n_layers, 2);
-  launch_pdl(k_commit_kv, grid, dim3(256), 0, s, st, kv, spb, is_draft);
+void launch_commit_kv(const StepState& st, KvStore tkv, KvStore dkv, int t_spb, int d_spb,
+                      cudaStream_t s) {
+  dim3 grid(st.B, std::max(tkv.n_layers, dkv.n_layers), 4);
+  launch_pdl(k_commit_kv, grid, dim3(256), 0, s, st, tkv, dkv, t_spb, d_spb);
 }
 
-void launch_advance(const StepState& st, cudaStream_t s) {
-  launch_pdl(k_advance, dim3(st.B), dim3(32), 0, s, st);
+void launch_copy_out(const CopyOut& c, cudaStream_t s) {
+  int most = 0;
+  for (int n : c.n) most = std::max(most, n);
+  if (most) launch_pdl(k_copy_out, dim3((most + 255) / 256), dim3(256), 0, s, c);
 }
 
 void launch_rope_table(float2* table, int n_pos, int hd, float theta, cudaStream_t s) {

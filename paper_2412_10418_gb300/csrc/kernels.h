@@ -51,9 +51,16 @@ struct StepState {
 };
 
 // elementwise / row kernels (T = float or __nv_bfloat16, the model dtype)
-// h = E[token]; x = h . g in the GEMM-input format; ss = 32-feature partial sums of h^2
-void launch_embed(int dtype, const RowDesc* rows, int R, const void* embed, int D, float* h,
-                  void* x, size_t plane, const void* g, float* ss, int ld_ss, cudaStream_t s);
+// Which rows a pass has: built by the host (prefill), or planned on the device from the state: draft
+// call j of the rollout (spb tail slots per beam), the verify pass, and the same of Step-1 round 2
+// (rows [x' (+ c_1 when j = 1)] or lh_j-1, and [x', c_1, lh_1..lh_d] of every prompt).
+enum PlanKind : int32_t { PLAN_HOST = 0, PLAN_DRAFT, PLAN_VERIFY, PLAN_S1_DRAFT, PLAN_S1_VERIFY };
+struct RowPlan { StepState st; int32_t kind, j, spb; };
+// rows[r] planned; h = E[token]; x = h . g in the GEMM-input format; ss = 32-feature partial sums
+// of h^2
+void launch_embed(int dtype, const RowPlan& p, RowDesc* rows, int R, const void* embed, int D,
+                  float* h, void* x, size_t plane, const void* g, float* ss, int ld_ss,
+                  cudaStream_t s);
 // out: GEMM-input activations (store_act format, hi/lo planes `plane` elements apart)
 void launch_rmsnorm(int dtype, const float* h, int R, int D, const void* gain, float eps,
                     void* out, size_t plane, const int32_t* gather, const float* head_w,
@@ -74,6 +81,7 @@ struct AttnArgs {
   int32_t* status;
   unsigned long long* stamp;   // in-graph launch timing record (LaunchStamp), or nullptr
   uint64_t wait_ns;            // limit of the tensor-core kernel's MMA waits (nanoseconds)
+  int32_t rows_late;           // 1: the kernel before the previous one writes the rows (layer 0)
 };
 int attn_chunk();
 int attn_max_chunks();
@@ -186,23 +194,25 @@ void launch_gemm_pair(const TcMaps& maps, const GemmArgs& a, const PairPlan& p, 
 // Message returned by cdsl_last_error(NULL) on this thread.
 void set_thread_error(const char* msg);
 
-// plans and the decision
-void launch_plan_draft(const StepState& st, int j, int tail_slots_per_beam, RowDesc* rows,
-                       cudaStream_t s);
-void launch_plan_verify(const StepState& st, RowDesc* rows, cudaStream_t s);
-// Step-1 round 2: draft call j (1..d) over [x' (+ c_1 when j = 1)] or lh_j-1, and the target
-// pass over [x', c_1, lh_1..lh_d] of every prompt
-void launch_plan_s1_draft(const StepState& st, int j, RowDesc* rows, cudaStream_t s);
-void launch_plan_s1_verify(const StepState& st, RowDesc* rows, cudaStream_t s);
-// commit = 0: decide only (n_b, rewards, b*, state, emission); 1: also allocate KV pages
+// the decision
+// commit = 0: decide only (n_b, rewards, b*, state, emission); 1: also allocate KV pages and, with a
+// Step-1 budget below 2, advance the prompts (lengths, tokens, next roots)
 void launch_select(const StepState& st, KvStore tkv, KvStore dkv, int commit, cudaStream_t s);
-// Step-1 round 2's decision: R(T + c_1 + x' + lh) >= r_t emits c_1, x' (state 3). ss / hw:
+// Step-1 round 2's decision (R(T + c_1 + x' + lh) >= r_t emits c_1, x', state 3) and the advance. ss / hw:
 // the target pass's final-norm and reward-head partial sums (rows ld_ss apart).
 void launch_select_s1(const StepState& st, KvStore tkv, KvStore dkv, const float* ss,
                       const float* hw, int norm_D, int ld_ss, float norm_eps, cudaStream_t s);
-void launch_commit_kv(const StepState& st, KvStore kv, int slots_per_beam, int is_draft,
+// the emitted tokens' K/V of both models to the prefix pages, and the step counters
+void launch_commit_kv(const StepState& st, KvStore tkv, KvStore dkv, int t_spb, int d_spb,
                       cudaStream_t s);
-void launch_advance(const StepState& st, cudaStream_t s);
+// 32-bit words copied to the caller's buffers, n[q] of each (0: not wanted)
+struct CopyOut {
+  static constexpr int N = 5;
+  uint32_t* dst[N];
+  const uint32_t* src[N];
+  int32_t n[N];
+};
+void launch_copy_out(const CopyOut& c, cudaStream_t s);
 void launch_rope_table(float2* table, int n_pos, int hd, float theta, cudaStream_t s);
 
 }  // namespace cdsl
