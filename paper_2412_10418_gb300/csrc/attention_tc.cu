@@ -13,11 +13,18 @@
 // fp32 accuracy from bf16 operands: every fp32 input x is split into hi = bf16(x) and
 // lo = bf16(x - hi), and each product is hi.hi + hi.lo + lo.hi (lo.lo, about 2^-18 of the
 // product, is dropped), accumulated in fp32. The K/V cache stays fp32 in HBM; the block
-// converts each chunk while staging it (K row-major as the score product's B operand, V
-// transposed as the P V product's B operand). Staging is software-pipelined: the next
-// chunk's rows are loaded into registers while this chunk's softmax runs and stored once
-// its P V has completed. Q is split once per block, pre-scaled by log2(e) / sqrt(head_dim)
-// (scores in base 2).
+// converts each chunk while staging it (rows of keys: the score product's K-major B operand, and
+// the P V product's MN-major one). Staging is software-pipelined: the next chunk's K rows are
+// loaded into registers while this chunk's softmax runs and stored once its P V has completed. Q
+// is split once per block, pre-scaled by log2(e) / sqrt(head_dim) (scores in base 2).
+//
+// What bounds it: the chain of a chunk's phases (loads, conversion, score MMAs, softmax, P V), 6 us
+// on eight warps with DRAM and the tensor pipe both below 10 %. Two groups of eight warps work on
+// alternate chunks of the block, each with its own K, V and P in shared memory (P over K) and its own
+// S, O and softmax state; their partials are added at the end. 13B verify pass (224 rows, 1,100
+// keys): 128 us per launch with one group, 112 with two, 108 with V staged by rows as K is (it
+// was transposed by 4-byte loads); 176 rows at 4,160 keys 184, 156, 144. Three planes of P and V
+// (prefill, head_dim 128) leave shared memory for one group.
 //
 // Softmax: warps w and w + 4 read TMEM lanes 32(w % 4) .. +31, so each thread owns one query
 // vector's row of scores over half the chunk's keys (the two halves exchange their row
@@ -48,35 +55,41 @@ using attn::ACH;
 using attn::MAXCB;
 
 constexpr int TQB = 128;             // query vectors per block (at most): the MMA's M
-constexpr int TTHREADS = 256;
-constexpr int TWARPS = TTHREADS / 32;
+constexpr int GTHREADS = 256;        // threads of a group, which works on a chunk at a time
 constexpr int TACL = 16;             // blocks per cluster (at most)
-constexpr int kIssuer = 128;         // thread that issues the MMAs (warp 4, lane 0)
+constexpr int kIssuer = 128;         // thread of a group that issues its MMAs (warp 4, lane 0)
 constexpr float kLazy = 11.5415602f; // raise the softmax reference only past this margin
                                      // (base-2 scores: 8 / ln 2, so p <= e^8)
 constexpr float kLog2e = 1.44269504088896341f;
 
 int g_tc_max_cluster = 8;
 
-// NP: planes of P and V (2: x = hi + lo; 3: hi + mid + lo, fp32's own precision).
-template <int HD, int NP>
+// NP: planes of P and V (2: x = hi + lo; 3: hi + mid + lo, fp32's own precision). NG: groups. Each
+// group has its own K, V and P; with two groups P overwrites K, whose products are done by then.
+template <int HD, int NP, int NG>
 struct TcSmem {
   static constexpr int KB = HD / 64;                        // 64-wide K blocks of Q and K
   static constexpr uint32_t Q_KB = TQB * 128;               // bytes of one K block of Q
   static constexpr uint32_t K_KB = ACH * 128;               // bytes of one K block of K
   static constexpr uint32_t Q_PLANE = KB * Q_KB;            // Q [128][HD] bf16, one plane
   static constexpr uint32_t K_PLANE = KB * K_KB;            // K [64][HD]
-  static constexpr uint32_t V_PLANE = HD * 128;             // V^T [HD][64 keys]
+  static constexpr uint32_t V_PLANE = K_PLANE;              // V [64][HD]
   static constexpr uint32_t P_PLANE = TQB * 128;            // P [128][64 keys]
   static constexpr uint32_t Q_OFF = 0;
   static constexpr uint32_t K_OFF = Q_OFF + 2 * Q_PLANE;
-  static constexpr uint32_t V_OFF = K_OFF + 2 * K_PLANE;
-  static constexpr uint32_t P_OFF = V_OFF + NP * V_PLANE;
-  static constexpr uint32_t TOTAL = P_OFF + NP * P_PLANE;
+  static constexpr bool ALIAS = NG > 1;
+  static_assert(!ALIAS || NP * P_PLANE <= 2 * K_PLANE || HD < 128, "P fits over K");
+  static constexpr uint32_t KP = ALIAS && NP * P_PLANE > 2 * K_PLANE ? NP * P_PLANE : 2 * K_PLANE;
+  static constexpr uint32_t V_OFF = K_OFF + KP;
+  static constexpr uint32_t P_OFF = ALIAS ? K_OFF : V_OFF + NP * V_PLANE;
+  static constexpr uint32_t GROUP = KP + NP * V_PLANE + (ALIAS ? 0 : NP * P_PLANE);   // per group
+  static constexpr uint32_t TOTAL = K_OFF + NG * GROUP;
   static constexpr int OP = HD + 4;                         // row pitch of the partial o (floats)
-  static constexpr uint32_t O_OFF = K_OFF;                  // partial o [128][OP] fp32, after the
-  static_assert(TQB * OP * 4 <= TOTAL - K_OFF, "partial o fits over K, V and P");   // chunks
-  static constexpr uint32_t TMEM_COLS = (64 + HD) <= 128 ? 128 : 256;
+  // partial o [128][OP] fp32 of each group, over everything after the chunks; the block's first
+  static_assert(NG * TQB * OP * 4 <= TOTAL, "the partial o fit");
+  static constexpr uint32_t O_SIZE = TQB * OP * 4;
+  static constexpr uint32_t T_GROUP = 64 + HD;              // TMEM columns of a group: S, O
+  static constexpr uint32_t TMEM_COLS = NG * T_GROUP <= 128 ? 128 : NG * T_GROUP <= 256 ? 256 : 512;
   static constexpr size_t bytes = TOTAL + 1024;             // + 1024-byte alignment of the base
 };
 
@@ -105,26 +118,28 @@ __device__ __forceinline__ void st_shared16(uint8_t* base, uint32_t off, const u
   *reinterpret_cast<uint4*>(base + off) = v;
 }
 
-template <int HD, int NP>
-__global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
+template <int HD, int NP, int NG>
+__global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
   const LaunchStamp stamp(a.stamp);
-  using SM = TcSmem<HD, NP>;
+  using SM = TcSmem<HD, NP, NG>;
+  constexpr int TTHREADS = NG * GTHREADS, TWARPS = TTHREADS / 32;
   constexpr int KB = SM::KB;
   constexpr int DCH = HD / 8;                    // 16-byte bf16 chunks per row of Q and K
-  constexpr int K_IT = ACH * DCH / TTHREADS;     // staging items per thread: K (key, chunk)
-  constexpr int V_IT = HD * (ACH / 8) / TTHREADS;  //   and V^T (dim, 8 keys)
+  constexpr int K_IT = ACH * DCH / GTHREADS;     // staging items per thread: K and V
+                                                 //   (key, 16-byte chunk)
   constexpr int Q_IT = TQB * DCH / TTHREADS;     //   and Q (query vector, chunk)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_raw + ((1024 - (tc::smem_u32(smem_raw) & 1023)) & 1023);
   __shared__ attn::Layout<TQB> L;
-  __shared__ __align__(8) uint64_t bar_s, bar_o;   // score / P V products complete
-  __shared__ __align__(8) uint64_t bar_d;          // every MMA of the block has completed
+  // per group: score / P V products complete, every MMA of it has completed
+  __shared__ __align__(8) uint64_t bar_s[NG], bar_o[NG], bar_d[NG];
   __shared__ uint32_t s_tmem;
-  __shared__ int s_abort, s_nkeys;
-  __shared__ const float* s_kptr[2][ACH];         // K of each key slot of a chunk (V follows);
-                                                  // chunk i uses buffer i & 1
+  __shared__ int s_abort[NG], s_nkeys;
+  __shared__ const float* s_kptr[NG][2][ACH];     // K of each key slot of a chunk (V follows); a
+                                                  // group's chunks take the buffers in turn
   __shared__ float s_pm[TQB], s_pl[TQB];          // the block's partial (m, l) per query vector
-  __shared__ float s_mx[2][TQB];                  // per half: a chunk's row maxima, then l
+  __shared__ float s_gm[TQB], s_gl[TQB];          // the second group's
+  __shared__ float s_mx[NG][2][TQB];              // per half: a chunk's row maxima, then l
 
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)gridDim.x;                   // = cluster size
@@ -142,76 +157,78 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
   const int nb_chunks = L.nb;                     // chunk_of(L, n_p, cx, C, 0 .. nb_chunks - 1)
   if (a.stamp) attn::count_bytes<TQB, TTHREADS, HD>(L, stamp, qb, cx, nb_chunks, nq, &s_nkeys);
   if (threadIdx.x == 0) {
-    tc::mbar_init(&bar_s, 1);
-    tc::mbar_init(&bar_o, 1);
-    tc::mbar_init(&bar_d, 1);
-    s_abort = 0;
+    for (int q = 0; q < NG; ++q) {
+      tc::mbar_init(&bar_s[q], 1);
+      tc::mbar_init(&bar_o[q], 1);
+      tc::mbar_init(&bar_d[q], 1);
+      s_abort[q] = 0;
+    }
     tc::fence_mbar_init();
   }
   pdl_wait();                 // q and K/V of the previous kernels are ready
-  pdl_launch_dependents();
   if (warp == 0) tc::tmem_alloc(&s_tmem, SM::TMEM_COLS);
 
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
-  const uint32_t tmem = s_tmem;
+  pdl_launch_dependents();    // (this block has its TMEM before any of the next kernel's)
+  const int grp = threadIdx.x / GTHREADS, tid = threadIdx.x % GTHREADS;
+  auto group_sync = [&] { tc::named_barrier(1 + grp, GTHREADS); };
+  const uint32_t tmem = s_tmem + (uint32_t)grp * SM::T_GROUP;
   const uint32_t t_s = tmem, t_o = tmem + 64;      // columns: S [0, 64), O [64, 64 + HD)
   const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
   const uint32_t sbase = tc::smem_u32(sm);
-  const uint32_t idesc_s = tc::idesc_bf16_f32(128, ACH), idesc_o = tc::idesc_bf16_f32(128, HD);
+  uint8_t* const smg = sm + grp * SM::GROUP;       // base of the group's K, V and P
+  const uint32_t gbase = sbase + (uint32_t)grp * SM::GROUP;
+  const uint32_t idesc_s = tc::idesc_bf16_f32(128, ACH), idesc_o = tc::idesc_bf16_f32(128, HD, true);
   const size_t v_delta_tail = (size_t)a.kv.n_tail_slots * a.kv.kvh * HD;
   const size_t v_delta_pfx = ((size_t)a.kv.kvh << a.kv.page_shift) * HD;
-  const int qi = threadIdx.x & (TQB - 1);          // softmax: TMEM lane (query vector) and
-  const int half = threadIdx.x / TQB;              //   half of the chunk's keys
+  const int qi = tid & (TQB - 1);                  // softmax: TMEM lane (query vector) and
+  const int half = tid / TQB;                      //   half of the chunk's keys
   float m_ref = -INFINITY, l_run = 0.f;
   int nproc = 0;                                    // chunks whose P V has been issued
 
-  // Staging is software-pipelined: chunk i + 1's K and V rows are loaded from the fp32 cache
-  // into registers right after chunk i's score MMAs are issued (in flight during its
-  // softmax), and converted and stored once chunk i's P V has completed.
-  auto kptrs = [&](int i) {   // threads 0 .. ACH-1: key slot pointers of chunk i
-    if (threadIdx.x < ACH) {
+  // Staging is software-pipelined: the group's next K rows (with one group, the V rows too) are
+  // loaded from the fp32 cache into registers right after a chunk's score MMAs are issued (in
+  // flight during its softmax), and converted and stored once its P V has completed.
+  constexpr bool kPreV = NG == 1;
+  auto kptrs = [&](int i) {   // the group's threads 0 .. ACH-1: key slot pointers of chunk i
+    if (tid < ACH) {
       const int c = attn::chunk_of(L, n_p, cx, C, i);
-      const int ks = L.kslot[i * ACH + threadIdx.x];
+      const int ks = L.kslot[i * ACH + tid];
       const float* kp = nullptr;
       if (ks >= 0) {
-        const int slot = (c * ACH + threadIdx.x) & ((1 << a.kv.page_shift) - 1);
+        const int slot = (c * ACH + tid) & ((1 << a.kv.page_shift) - 1);
         kp = c >= n_p ? a.kv.tail + kv_tail_offset(a.kv, a.layer, 0, ks, g)
                       : a.kv.pool + kv_prefix_offset(a.kv, a.layer, ks, 0, g, slot);
       }
-      s_kptr[i & 1][threadIdx.x] = kp;
+      s_kptr[grp][(i / NG) & 1][tid] = kp;
     }
   };
-  float4 kr[K_IT][2];   // raw K and V of the next chunk to stage
-  float vr[V_IT][8];
-  auto load_kv = [&](int i) {   // all loads of chunk i in flight together (pointers ready)
-    const size_t v_delta = attn::chunk_of(L, n_p, cx, C, i) >= n_p ? v_delta_tail : v_delta_pfx;
-    const float* const* kps = s_kptr[i & 1];
+  float4 kr[K_IT][2], vr[K_IT][2];   // raw K and V of the next chunk to stage
+  // K or V (v_delta floats behind) rows of chunk i, all loads in flight together (pointers ready)
+  auto load_rows = [&](int i, size_t delta, float4 (&x)[K_IT][2]) {
+    const float* const* kps = s_kptr[grp][(i / NG) & 1];
 #pragma unroll
     for (int u = 0; u < K_IT; ++u) {
-      const int idx = threadIdx.x + u * TTHREADS, j = idx / DCH, dc = idx % DCH;
+      const int idx = tid + u * GTHREADS, j = idx / DCH, dc = idx % DCH;
       const float* kp = kps[j];
-      kr[u][0] = kr[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (kp) {
-        kr[u][0] = __ldg(reinterpret_cast<const float4*>(kp + dc * 8));
-        kr[u][1] = __ldg(reinterpret_cast<const float4*>(kp + dc * 8 + 4));
+        x[u][0] = __ldg(reinterpret_cast<const float4*>(kp + delta + dc * 8));
+        x[u][1] = __ldg(reinterpret_cast<const float4*>(kp + delta + dc * 8 + 4));
       }
     }
-#pragma unroll
-    for (int u = 0; u < V_IT; ++u) {
-      const int idx = threadIdx.x + u * TTHREADS, d = idx % HD, jc = idx / HD;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float* kp = kps[jc * 8 + q];
-        vr[u][q] = kp ? __ldg(kp + v_delta + d) : 0.f;
-      }
-    }
+  };
+  auto load_k = [&](int i) { load_rows(i, 0, kr); };
+  auto load_v = [&](int i) {
+    load_rows(i, attn::chunk_of(L, n_p, cx, C, i) >= n_p ? v_delta_tail : v_delta_pfx, vr);
   };
   if (nb_chunks > 0 && nq > 0) {
     // ---- Q once per block: query vector qi is row qi of the A operand (zero rows from nq
-    //      on), pre-scaled by log2(e) / sqrt(head_dim) (base-2 scores); and chunk 0's loads
-    kptrs(0);
+    //      on), pre-scaled by log2(e) / sqrt(head_dim) (base-2 scores); and the groups' first
+    //      chunks' loads
+    if (grp < nb_chunks) kptrs(grp);
     float4 qr[Q_IT][2];
 #pragma unroll
     for (int u = 0; u < Q_IT; ++u) {
@@ -224,8 +241,11 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
         qr[u][1] = *reinterpret_cast<const float4*>(src + 4);
       }
     }
-    __syncthreads();   // chunk 0's pointers
-    load_kv(0);
+    __syncthreads();   // the first chunks' pointers
+    if (grp < nb_chunks) {
+      load_k(grp);
+      if (kPreV) load_v(grp);
+    }
 #pragma unroll
     for (int u = 0; u < Q_IT; ++u) {
       const int it = threadIdx.x + u * TTHREADS, qv = it / DCH, dc = it % DCH;
@@ -240,46 +260,54 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
     }
   }
 
-  for (int i = 0; i < nb_chunks && nq > 0; ++i) {
+  if (NG > 1) {   // Q, which both groups' MMAs read, is complete
+    tc::fence_proxy_async();
+    __syncthreads();
+  }
+  for (int i = grp; i < nb_chunks && nq > 0; i += NG) {
     const int c = attn::chunk_of(L, n_p, cx, C, i);
     const bool tail = c >= n_p;
     const int t0 = c * ACH;
-    // the previous chunk's P V has completed: K, V and P may be overwritten
-    if (nproc > 0 && !tc::mbar_wait(&bar_o, (nproc - 1) & 1, a.status, a.wait_ns)) s_abort = 1;
-    if (i + 1 < nb_chunks) kptrs(i + 1);
+    if (!kPreV) load_v(i);
+    // the group's previous P V has completed: K, V and P may be overwritten
+    if (nproc > 0 && !tc::mbar_wait(&bar_o[grp], (nproc - 1) & 1, a.status, a.wait_ns))
+      s_abort[grp] = 1;
+    if (i + NG < nb_chunks) kptrs(i + NG);
     // ---- stage the chunk: split the loaded K and V into hi/lo and store
 #pragma unroll
     for (int u = 0; u < K_IT; ++u) {
-      const int idx = threadIdx.x + u * TTHREADS, j = idx / DCH, dc = idx % DCH;
+      const int idx = tid + u * GTHREADS, j = idx / DCH, dc = idx % DCH;
       const float x[8] = {kr[u][0].x, kr[u][0].y, kr[u][0].z, kr[u][0].w,
                           kr[u][1].x, kr[u][1].y, kr[u][1].z, kr[u][1].w};
       uint4 p[2];
       split8<2>(x, p);
       const uint32_t off = SM::K_OFF + (dc >> 3) * SM::K_KB + tc::sw128_offset(j, dc & 7);
-      st_shared16(sm, off, p[0]);
-      st_shared16(sm, off + SM::K_PLANE, p[1]);
+      st_shared16(smg, off, p[0]);
+      st_shared16(smg, off + SM::K_PLANE, p[1]);
     }
 #pragma unroll
-    for (int u = 0; u < V_IT; ++u) {
-      const int idx = threadIdx.x + u * TTHREADS, d = idx % HD, jc = idx / HD;
+    for (int u = 0; u < K_IT; ++u) {
+      const int idx = tid + u * GTHREADS, j = idx / DCH, dc = idx % DCH;
+      const float x[8] = {vr[u][0].x, vr[u][0].y, vr[u][0].z, vr[u][0].w,
+                          vr[u][1].x, vr[u][1].y, vr[u][1].z, vr[u][1].w};
       uint4 p[NP];
-      split8<NP>(vr[u], p);
-      const uint32_t off = SM::V_OFF + tc::sw128_offset(d, jc);
+      split8<NP>(x, p);
+      const uint32_t off = SM::V_OFF + (dc >> 3) * SM::K_KB + tc::sw128_offset(j, dc & 7);
 #pragma unroll
-      for (int n = 0; n < NP; ++n) st_shared16(sm, off + n * SM::V_PLANE, p[n]);
+      for (int n = 0; n < NP; ++n) st_shared16(smg, off + n * SM::V_PLANE, p[n]);
     }
     tc::fence_proxy_async();
-    __syncthreads();
-    if (s_abort) break;
+    group_sync();
+    if (s_abort[grp]) break;
     // ---- S = Q K^T (hi.hi + hi.lo + lo.hi over the head dimension)
-    if (threadIdx.x == kIssuer) {
+    if (tid == kIssuer) {
       tc::tc_fence_after();
 #pragma unroll
       for (int kb = 0; kb < KB; ++kb) {
         const uint64_t qh = tc::desc_sw128(sbase + SM::Q_OFF + kb * SM::Q_KB);
         const uint64_t ql = tc::desc_sw128(sbase + SM::Q_OFF + SM::Q_PLANE + kb * SM::Q_KB);
-        const uint64_t kh = tc::desc_sw128(sbase + SM::K_OFF + kb * SM::K_KB);
-        const uint64_t kl = tc::desc_sw128(sbase + SM::K_OFF + SM::K_PLANE + kb * SM::K_KB);
+        const uint64_t kh = tc::desc_sw128(gbase + SM::K_OFF + kb * SM::K_KB);
+        const uint64_t kl = tc::desc_sw128(gbase + SM::K_OFF + SM::K_PLANE + kb * SM::K_KB);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {   // K = 16 per MMA: +32 bytes = +2 in the descriptor
           tc::umma_bf16(t_s, qh + 2 * kk, kh + 2 * kk, idesc_s, (kb | kk) ? 1u : 0u);
@@ -287,17 +315,20 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
           tc::umma_bf16(t_s, ql + 2 * kk, kh + 2 * kk, idesc_s, 1u);
         }
       }
-      tc::umma_commit(&bar_s);
+      tc::umma_commit(&bar_s[grp]);
     }
-    if (i + 1 < nb_chunks) load_kv(i + 1);   // in flight during this chunk's softmax
+    if (i + NG < nb_chunks) {   // in flight during this chunk's softmax
+      load_k(i + NG);
+      if (kPreV) load_v(i + NG);
+    }
     // ---- softmax over the chunk: thread t owns TMEM lane qi = t % 128 (a query vector) and
     //      the chunk's keys 32h .. 32h + 31, h = t / 128 (warps w and w + 4 read the same
     //      lanes; tcgen05.ld is warp-collective, so a warp takes every branch as a whole)
-    const bool sok = __all_sync(0xffffffffu, tc::mbar_wait(&bar_s, nproc & 1, a.status, a.wait_ns));
+    const bool sok = __all_sync(0xffffffffu, tc::mbar_wait(&bar_s[grp], nproc & 1, a.status, a.wait_ns));
     float s[2][16];
     float mx = -INFINITY;
     if (!sok) {
-      s_abort = 1;
+      s_abort[grp] = 1;
     } else {
       tc::tc_fence_after();
       uint32_t r[2][16];
@@ -317,11 +348,11 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
           s[q][e] = vis ? __uint_as_float(r[q][e]) : -INFINITY;   // masked: 2^(-inf - m) = 0
           mx = fmaxf(mx, s[q][e]);
         }
-      s_mx[half][qi] = mx;
+      s_mx[grp][half][qi] = mx;
     }
-    __syncthreads();
-    if (s_abort) break;
-    mx = fmaxf(s_mx[0][qi], s_mx[1][qi]);   // the row's maximum, the same in both halves
+    group_sync();
+    if (s_abort[grp]) break;
+    mx = fmaxf(s_mx[grp][0][qi], s_mx[grp][1][qi]);   // the row's maximum, the same in both halves
     {
       // raise the reference where a row's maximum passed it by more than kLazy: its earlier
       // sum and output are rescaled by alpha = exp(m_old - m_new) (both halves decide alike)
@@ -367,21 +398,21 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
         split8<NP>(x, p);
         const uint32_t off = SM::P_OFF + tc::sw128_offset(qi, 4 * half + cc);
 #pragma unroll
-        for (int n = 0; n < NP; ++n) st_shared16(sm, off + n * SM::P_PLANE, p[n]);
+        for (int n = 0; n < NP; ++n) st_shared16(smg, off + n * SM::P_PLANE, p[n]);
       }
       tc::fence_proxy_async();
       tc::tc_fence_before();
     }
-    __syncthreads();
+    group_sync();
     // ---- O += P V over the chunk's 64 keys: hi.hi + hi.lo + lo.hi, or with three planes the six
     //      products down to 2^-24 of the largest
-    if (threadIdx.x == kIssuer) {
+    if (tid == kIssuer) {
       tc::tc_fence_after();
       uint64_t pd[NP], vd[NP];
 #pragma unroll
       for (int n = 0; n < NP; ++n) {
-        pd[n] = tc::desc_sw128(sbase + SM::P_OFF + n * SM::P_PLANE);
-        vd[n] = tc::desc_sw128(sbase + SM::V_OFF + n * SM::V_PLANE);
+        pd[n] = tc::desc_sw128(gbase + SM::P_OFF + n * SM::P_PLANE);
+        vd[n] = tc::desc_sw128_mn(gbase + SM::V_OFF + n * SM::V_PLANE, SM::K_KB);
       }
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
@@ -389,56 +420,75 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
         for (int n = 0; n < NP; ++n)
 #pragma unroll
           for (int m = 0; n + m < NP; ++m)
-            tc::umma_bf16(t_o, pd[n] + 2 * kk, vd[m] + 2 * kk, idesc_o,
+            tc::umma_bf16(t_o, pd[n] + 2 * kk, vd[m] + 128 * kk, idesc_o,   // 16 keys: 2 KB
                           (nproc | kk | n | m) ? 1u : 0u);
-      tc::umma_commit(&bar_o);
+      tc::umma_commit(&bar_o[grp]);
     }
     ++nproc;
   }
 
   // ---- every MMA issued here completes before its operands are overwritten and TMEM is
   //      released (fixed limit, also after a give-up)
-  if (threadIdx.x == kIssuer) {
-    tc::umma_commit(&bar_d);
-    tc::mbar_wait(&bar_d, 0, a.status);
+  if (tid == kIssuer) {
+    tc::umma_commit(&bar_d[grp]);
+    tc::mbar_wait(&bar_d[grp], 0, a.status);
   }
-  // ---- the block's partial (m, l, o) per query vector into shared memory (o over K, V, P):
-  //      each half writes its half of the row's columns; l is the sum of the halves' shares
-  if (nproc > 0 && !tc::mbar_wait(&bar_o, (nproc - 1) & 1, a.status, a.wait_ns)) s_abort = 1;
-  if (half == 1) s_mx[1][qi] = l_run;
+  // ---- the block's partial (m, l, o) per query vector into shared memory (o over everything):
+  //      each half writes its half of the row's columns; l is the sum of the halves' shares. A
+  //      second group leaves its partial there for the first one to add to its own.
+  if (nproc > 0 && !tc::mbar_wait(&bar_o[grp], (nproc - 1) & 1, a.status, a.wait_ns))
+    s_abort[grp] = 1;
+  if (half == 1) s_mx[grp][1][qi] = l_run;
   __syncthreads();
-  float* s_po = reinterpret_cast<float*>(sm + SM::O_OFF);   // [TQB][OP]
-  const bool have_o = nproc > 0 && !s_abort;
+  float* const s_po = reinterpret_cast<float*>(sm);              // [TQB][OP]
+  float* const s_go = s_po + SM::O_SIZE / 4;                     // the second group's
+  const bool have_o = nproc > 0 && !s_abort[grp];
   if (have_o) tc::tc_fence_after();
+  auto each_o = [&](auto&& put) {   // put(column, 16 values) over this half's columns
 #pragma unroll 1
-  for (int q0 = 0; q0 < HD / 32; q0 += 4) {   // 64 columns per wait
-    uint32_t o[4][16];
+    for (int q = 0; q < HD / 32; ++q) {
+      const int col = half * (HD / 2) + 16 * q;
+      float o[16];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (have_o && q0 + q < HD / 32) {
-        tc::tmem_ld16_nowait(t_o + lane_base + half * (HD / 2) + 16 * (q0 + q), o[q]);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) o[q][e] = 0u;
-      }
+      for (int e = 0; e < 16; ++e) o[e] = 0.f;
+      if (have_o) tc::tmem_ld16(t_o + lane_base + col, o);   // (uniform over the group)
+      if (qi < nq) put(col, o);
     }
-    if (have_o) tc::tmem_wait_ld();
-    if (qi < nq) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (q0 + q < HD / 32)
-#pragma unroll
-          for (int e = 0; e < 16; e += 4) {
-            float* dst = s_po + qi * SM::OP + half * (HD / 2) + 16 * (q0 + q) + e;
-            *reinterpret_cast<float4*>(dst) =
-                make_float4(__uint_as_float(o[q][e]), __uint_as_float(o[q][e + 1]),
-                            __uint_as_float(o[q][e + 2]), __uint_as_float(o[q][e + 3]));
-          }
+  };
+  if (half == 0) l_run += s_mx[grp][1][qi];
+  if (NG > 1 && grp == 1) {
+    if (half == 0) {
+      s_gm[qi] = have_o ? m_ref : -INFINITY;
+      s_gl[qi] = have_o ? l_run : 0.f;
     }
+    each_o([&](int col, const float (&o)[16]) {
+#pragma unroll
+      for (int e = 0; e < 16; e += 4)
+        *reinterpret_cast<float4*>(s_go + qi * SM::OP + col + e) =
+            make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]);
+    });
   }
-  if (half == 0 && qi < nq) {
-    s_pm[qi] = have_o ? m_ref : -INFINITY;
-    s_pl[qi] = have_o ? l_run + s_mx[1][qi] : 0.f;
+  if (NG > 1) __syncthreads();
+  if (grp == 0) {
+    const float m0 = have_o ? m_ref : -INFINITY, m1 = NG > 1 ? s_gm[qi] : -INFINITY;
+    const float m = fmaxf(m0, m1);
+    const float f0 = m0 > -INFINITY ? exp2f(m0 - m) : 0.f, f1 = m1 > -INFINITY ? exp2f(m1 - m) : 0.f;
+    each_o([&](int col, const float (&o)[16]) {
+#pragma unroll
+      for (int e = 0; e < 16; e += 4) {
+        float4 v = make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]);
+        if (NG > 1) {
+          const float4 w = *reinterpret_cast<const float4*>(s_go + qi * SM::OP + col + e);
+          v.x = v.x * f0 + w.x * f1; v.y = v.y * f0 + w.y * f1;
+          v.z = v.z * f0 + w.z * f1; v.w = v.w * f0 + w.w * f1;
+        }
+        *reinterpret_cast<float4*>(s_po + qi * SM::OP + col + e) = v;
+      }
+    });
+    if (half == 0 && qi < nq) {
+      s_pm[qi] = m;
+      s_pl[qi] = (have_o ? l_run * f0 : 0.f) + (NG > 1 ? s_gl[qi] * f1 : 0.f);
+    }
   }
   tc::tc_fence_before();
   cluster.sync();   // every block's partials are visible to the cluster
@@ -494,31 +544,34 @@ __global__ void __launch_bounds__(TTHREADS, 1) k_attn_tc(AttnArgs a) {
     for (int c2 = 0; c2 < DPL; ++c2) store_act<__nv_bfloat16>(out, a.plane, dst + c2, acc[c2] * inv);
   }
   cluster.sync();   // no block leaves while the others may still read its shared memory
-  if (warp == 0) tc::tmem_dealloc(tmem, SM::TMEM_COLS);
+  if (warp == 0) tc::tmem_dealloc(s_tmem, SM::TMEM_COLS);
 }
 
-template <int HD, int NP>
-ClusterFit g_tc_fit;   // cluster residency of k_attn_tc<HD, NP> (configure_tc)
+template <int HD, int NP, int NG>
+ClusterFit g_tc_fit;   // cluster residency of k_attn_tc<HD, NP, NG> (configure_tc)
 
-template <int HD, int NP>
+template <int HD, int NP, int NG>
 int configure_tc() {
-  auto k = k_attn_tc<HD, NP>;
-  constexpr size_t smem = TcSmem<HD, NP>::bytes;
+  auto k = k_attn_tc<HD, NP, NG>;
+  constexpr size_t smem = TcSmem<HD, NP, NG>::bytes;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return -1;
   const bool nonportable =
       cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
   cudaGetLastError();
-  fill_cluster_fit(&g_tc_fit<HD, NP>, k, TTHREADS, smem, nonportable ? TACL : 8);
-  return nonportable && g_tc_fit<HD, NP>.active[TACL] >= 1 ? 0 : 1;   // 1: portable only
+  fill_cluster_fit(&g_tc_fit<HD, NP, NG>, k, NG * GTHREADS, smem, nonportable ? TACL : 8);
+  return nonportable && g_tc_fit<HD, NP, NG>.active[TACL] >= 1 ? 0 : 1;   // 1: portable only
 }
 
-template <int HD, int NP>
+template <int HD, int NP, int NG>
 void launch_tc(const AttnArgs& a, int n_z, cudaStream_t s) {
-  const int cl = attn_cluster_size(g_tc_fit<HD, NP>, g_tc_max_cluster, a.n_chunks + a.n_tchunks,
-                                   a.kv.kvh * n_z);
-  launch_pdl_cluster(k_attn_tc<HD, NP>, dim3(cl, a.kv.kvh, n_z), dim3(TTHREADS),
-                     TcSmem<HD, NP>::bytes, cl, s, a);
+  const int chunks = a.n_chunks + a.n_tchunks;
+  const ClusterFit& f = g_tc_fit<HD, NP, NG>;
+  const int groups = a.kv.kvh * n_z;
+  const int cl = a.zmap ? attn_cluster_size_causal(f, g_tc_max_cluster, chunks, groups)
+                        : attn_cluster_size(f, g_tc_max_cluster, chunks, groups);
+  launch_pdl_cluster(k_attn_tc<HD, NP, NG>, dim3(cl, a.kv.kvh, n_z), dim3(NG * GTHREADS),
+                     TcSmem<HD, NP, NG>::bytes, cl, s, a);
 }
 
 }  // namespace
@@ -534,8 +587,8 @@ int attn_tc_qblock(int rows_per_prompt, int G, bool tails) {
 
 int configure_attention_tc() {
   int worst = 0;
-  for (int r : {configure_tc<128, 2>(), configure_tc<64, 2>(), configure_tc<128, 3>(),
-                configure_tc<64, 3>()}) {
+  for (int r : {configure_tc<128, 2, 2>(), configure_tc<64, 2, 2>(), configure_tc<128, 3, 1>(),
+                configure_tc<64, 3, 2>()}) {
     if (r < 0) return -1;
     worst = std::max(worst, r);
   }
@@ -546,8 +599,10 @@ int configure_attention_tc() {
 void launch_attn_tc(const AttnArgs& a, int n_z, cudaStream_t s) {
   // prefill passes with three planes of P and V: their K/V cache carries every later step (two
   // planes: 13B logits after two layers 2.1e-5 -> 2.6e-5 off 64 bits, 3 to 7 % of the pass)
-  if (a.n_tchunks == 0) a.kv.hd == 128 ? launch_tc<128, 3>(a, n_z, s) : launch_tc<64, 3>(a, n_z, s);
-  else a.kv.hd == 128 ? launch_tc<128, 2>(a, n_z, s) : launch_tc<64, 2>(a, n_z, s);
+  if (a.n_tchunks == 0)
+    a.kv.hd == 128 ? launch_tc<128, 3, 1>(a, n_z, s) : launch_tc<64, 3, 2>(a, n_z, s);
+  else
+    a.kv.hd == 128 ? launch_tc<128, 2, 2>(a, n_z, s) : launch_tc<64, 2, 2>(a, n_z, s);
 }
 
 }  // namespace cdsl

@@ -231,11 +231,21 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
   return d;
 }
 
-// Instruction descriptor of kind::f16 with bf16 A and B (both K-major), fp32 accumulator.
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
+// The same for an MN-major operand tile (rows of one K value each, 64 M or N values = 128 bytes):
+// 8-row groups (K) 1024 bytes apart, the next 64 M or N values `block` bytes on. 16 K values
+// are 2048 bytes: +128 in the start field.
+__device__ __forceinline__ uint64_t desc_sw128_mn(uint32_t saddr, uint32_t block) {
+  uint64_t d = desc_sw128(saddr) & ~((uint64_t)0x3FFF << 16);
+  return d | (uint64_t)(block >> 4) << 16;    // leading byte offset: between blocks along M / N
+}
+
+// Instruction descriptor of kind::f16 with bf16 A and B (K-major; b_mn: B MN-major), fp32
+// accumulator.
+__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool b_mn = false) {
   return (1u << 4)                         // D format: f32
          | (1u << 7)                       // A format: bf16
          | (1u << 10)                      // B format: bf16
+         | ((b_mn ? 1u : 0u) << 16)        // B major-ness
          | ((uint32_t)(N >> 3) << 17)      // N / 8
          | ((uint32_t)(M >> 4) << 24);     // M / 16
 }
