@@ -1,4 +1,5 @@
-"""The CUDA-core GEMM and the no-scratch GEMV at the edges of their tiles and splits.
+"""The CUDA-core GEMM, the logits row statistics and the no-scratch GEMV at the edges of their tiles
+and splits.
 
 GEMM, through whole passes against the oracle: K ranges of less than one 32-wide step, with a
 remainder and of many steps (d_ffn is the down projection's K), row counts around its 32-row
@@ -32,6 +33,17 @@ def test_k_ranges_and_row_tiles(dtype, tol, d_ffn, batch, k, d):
     wl = synth.scaled(synth.TINY, dtype=dtype, target=mk(2, 192, 3, 1), draft=mk(1, 64, 1, 1),
                       batch=batch, k=k, d=d, prompt_len=37, max_new=6, reward_head=True)
     run_parity(make_setup(wl), steps=2, tol=tol, tol_r=tol)
+
+
+@pytest.mark.parametrize("vocab,batch,k", [(16, 1, 16), (8, 2, 3), (512, 3, 16), (4104, 6, 5)])
+def test_row_statistics_slices(vocab, batch, k):
+    """A logits row over clusters of eight, four, two and one blocks (verify rows 2 k batch): more
+    beams than logits in a slice, empty slices, uneven ones."""
+    mk = lambda: synth.ModelShape(n_layers=1, d_model=128, n_heads=2, n_kv_heads=1, d_ffn=96,
+                                  vocab=vocab)
+    wl = synth.scaled(synth.TINY, target=mk(), draft=mk(), batch=batch, k=k, d=1, prompt_len=5,
+                      max_new=6, n_keywords=2)
+    run_parity(make_setup(wl), steps=2, tol=1e-4, tol_r=1e-4)
 
 
 @pytest.mark.parametrize("R,K,N", [(1, 8, 1), (2, 264, 7), (3, 2056, 305), (4, 1024, 1217),
