@@ -21,9 +21,9 @@
 // most kSegKb blocks (2.2e-6), into two TMEM accumulator sets in turn; the epilogue warps add each
 // finished segment to fp32 sums in their registers (rounded to nearest) while the next one
 // accumulates (k_gemm_pair<.., true>). A K range of one segment is finished straight from TMEM
-// (<.., false>), and so are gate/up tiles of more than 128 rows, whose two accumulators leave
-// TMEM no room for a second set: one chain, for K up to kWideKb blocks (13B gate/up, 224 rows: 88
-// us against 115; the kernel before had the same chain there). Where TMEM has room (planes == 2)
+// (<.., false>), and so are gate/up and QKV tiles of more than 128 rows, whose two accumulators
+// leave TMEM no room for a second set: one chain, for gate/up of up to kWideKb blocks (13B, 224
+// rows: 88 us against 115; the kernel before had the same chain there), for QKV of kWideQkvKb. Where TMEM has room (planes == 2)
 // the lo plane accumulates apart, which halves a chain's truncations. 13B logits after two layers,
 // against 64 bits: 2.1e-5 (the kernel before: 2.7e-5; one chain per tile in all shapes: 3.3e-5).
 //
@@ -60,7 +60,8 @@ constexpr int kThreads = 64 + kEpThreads;
 constexpr int kGroups = kEpWarps / 4;   // warps that share 32 TMEM lanes
 constexpr int kChunks = 16 / kGroups;   // groups of 16 columns a warp sums
 constexpr int kSegKb = 16;           // 64-wide K blocks per accumulation chain (at most)
-constexpr int kWideKb = 80;          //   and of a tile's one chain that fills TMEM
+constexpr int kWideKb = 80;          //   and of a tile's one chain that fills TMEM: gate/up,
+constexpr int kWideQkvKb = 24;       //   QKV
 constexpr int kNMax = 256;
 constexpr int kSplitMax = 4;         // pairs per cluster (8 CTAs: the portable cluster size)
 constexpr size_t kSmemMax = 216 * 1024;   // dynamic shared memory a plan may use
@@ -454,17 +455,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if constexpr (MT == 2) load_sums(d + N + c, lo, y1);
             finish_sums<MODE>(a, tm, L, r0, c, rows, y0, MT == 2 ? y1 : y0, s_rs, s_qkv);
           }
-        } else {   // the partial tile to shared memory: [accumulator][row][128 features]
-          for (int c = cg * 16; c < rows; c += 16 * kGroups) {
-#pragma unroll
-            for (int m = 0; m < MT; ++m) {
-              float y[16];
-              load_sums(d + m * N + c, lo, y);
-#pragma unroll
-              for (int i = 0; i < 16; ++i) part[(size_t)(m * N + c + i) * 128] = y[i];
-            }
-          }
-        }
+        }   // (split K: below, straight from TMEM)
         tc::tc_fence_before();
         __syncwarp();
         if (lane == 0) tc::mbar_arrive_cluster(acce0 + 8u * (uint32_t)buf);
@@ -524,19 +515,41 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   if (S > 1) {
-    // ---- split K (one tile per cluster): CTA q of each half finishes rows
-    //      [q rows / S, (q + 1) rows / S) of its 128 weight rows
+    // ---- split K (one tile per cluster): the partial tiles go to shared memory, [accumulator][row]
+    //      [128 features], and CTA q of each half finishes rows [q n / S, (q + 1) n / S) of its 128
+    //      weight rows -- in two rounds of half the columns each where a partial tile does not
+    //      fit (p.rounds)
     const bool gave_up =
         warp >= 2 ? tc::named_barrier_or(1, kEpThreads, s_abort != 0) : true;
-    tc::cluster_arrive();   // this CTA's partial is complete (release)
-    tc::cluster_wait();     // every CTA's is (acquire)
-    if (!gave_up) {
-      const int quarter = warp & 3, cg = (warp - 2) >> 2;
-      const int tm = cid / NT, tn = cid % NT;
-      const int r0 = tn * N, rows = min(N, a.R - r0);
-      const int ra = q * rows / S, rb = (q + 1) * rows / S;
-      const int L = half * 128 + quarter * 32 + lane;
-      const uint32_t mine = tc::smem_u32(smem) + (quarter * 32 + lane) * 4;
+    const int quarter = warp & 3, cg = (warp - 2) >> 2;
+    const int tm = cid / NT, tn = cid % NT;
+    const int r0 = tn * N, rows = min(N, a.R - r0), NH = N / p.rounds;
+    const int L = half * 128 + quarter * 32 + lane;
+    const uint32_t mine = tc::smem_u32(smem) + (quarter * 32 + lane) * 4;
+    for (int rd = 0; rd < p.rounds; ++rd) {
+      const int b0 = rd * NH, n = max(0, min(rows - b0, NH));   // this round's columns
+      if (rd > 0) {   // the previous round's partials have been read
+        tc::cluster_arrive();
+        tc::cluster_wait();
+      }
+      if (!kSeg && !gave_up) {
+        float* const part = reinterpret_cast<float*>(smem) + quarter * 32 + lane;
+        const uint32_t d = tmem + ((uint32_t)(quarter * 32) << 16);
+        tc::tc_fence_after();
+        for (int c = cg * 16; c < n; c += 16 * kGroups) {
+#pragma unroll
+          for (int m = 0; m < MT; ++m) {
+            float y[16];
+            load_sums(d + m * N + b0 + c, lo, y);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) part[(size_t)(m * NH + c + i) * 128] = y[i];
+          }
+        }
+      }
+      tc::cluster_arrive();   // this CTA's partial is complete (release)
+      tc::cluster_wait();     // every CTA's is (acquire)
+      if (gave_up) continue;
+      const int ra = q * n / S, rb = (q + 1) * n / S;
       for (int c = ra + cg * 8; c < rb; c += 8 * kGroups) {
         float y0[8], y1[8];
 #pragma unroll
@@ -547,10 +560,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int i = 0; i < 8; ++i) {
             const int ci = min(i, rb - 1 - c) * 512;   // (past the share: any row, unused)
             y0[i] += tc::ld_cluster_f32(src + ci);
-            if constexpr (MT == 2) y1[i] += tc::ld_cluster_f32(src + N * 512 + ci);
+            if constexpr (MT == 2) y1[i] += tc::ld_cluster_f32(src + NH * 512 + ci);
           }
         }
-        finish_rows<MODE, 8>(a, tm, L, r0 + c, min(8, rb - c), y0, y1, s_rs + c, s_qkv + c);
+        finish_rows<MODE, 8>(a, tm, L, r0 + b0 + c, min(8, rb - c), y0, y1, s_rs + b0 + c,
+                             s_qkv + (MODE == EPI_QKV ? b0 + c : 0));
       }
     }
   }
@@ -623,28 +637,34 @@ PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt
       // chain where the tile's accumulators leave TMEM no room for it
       const int nkb = (KBT + S - 1) / S;
       const bool wide = MT * N > 256, seg = nkb > kSegKb && !wide;
-      if (wide && (mode != EPI_SWIGLU || nkb <= kSegKb || nkb > kWideKb)) continue;
+      if (wide && (nkb <= kSegKb ? S == 1 : nkb > (mode == EPI_SWIGLU ? kWideKb : kWideQkvKb)))
+        continue;
       // short chains keep lo apart rather than a second set where TMEM has no room for both
       const int bufs = wide || (!seg && (waves == 1 || 4 * MT * N > 512)) ? 1 : 2;
       const int stages = (int)std::min<size_t>(kStagesMax, (kSmemMax - 1024) / stage);
-      if (S > 1 && (size_t)stages * stage < (size_t)MT * N * 512) continue;
+      // a split's partial tiles reuse the stages, in two rounds if need be
+      const size_t part = (size_t)MT * N * 512, room = (size_t)stages * stage;
+      const int rounds = S == 1 || part <= room ? 1 : 2;
+      if (S > 1 && (part > rounds * room || (rounds == 2 && seg))) continue;
       const int planes = 2 * bufs * MT * N <= 512 ? 2 : 1;
-      // Estimated clocks, fitted to 1,900 measured plans (19 projection shapes of the 7B, 13B,
-      // 1B and small models, 66 to 1024 rows; the chosen plan is on average 1.2 % slower than
-      // the fastest of its shape): a K block costs the MMAs or the fetch of its operands (33
-      // bytes per clock and SM), the launch at least its weights at 19 bytes per clock and
-      // active SM; the last tile's epilogue is never hidden, the earlier ones' only where a
-      // second accumulator set fills meanwhile; a split adds the exchange of the partials.
+      // Estimated clocks, fitted to 1,500 measured plans (19 projection shapes of the 7B, 13B,
+      // 1B and small models, 72 to 1024 rows; the chosen plan is on average 0.9 % slower than
+      // the fastest of its shape): a K block costs the MMAs or the fetch of its operands (36
+      // bytes per clock and SM, 5,250 in all), the launch at least its weights at 22 bytes per
+      // clock and active SM; the last tile's epilogue is never hidden, the earlier ones' only
+      // where a second accumulator set fills meanwhile; a split adds the exchange of the
+      // partials, each CTA some of the launch.
       const int ctas = clusters * 2 * S;
-      const double kb = std::max(4.8 * MT * N, stage / 33.0), ep = 15.0 * MT * N;
+      const double kb = std::max(4.1 * MT * N, stage * std::max(1 / 36.5, ctas / 5250.0));
+      const double ep = 20.0 * MT * N;
       double cost = (double)waves * nkb * kb;
-      cost = std::max(cost, 2.0 * n_virtual * K / (19.0 * ctas)) + (20.0 + 0.04 * N) * ctas;
-      if (seg) cost += 2300;
+      cost = std::max(cost, 2.0 * n_virtual * K / (22.0 * ctas)) + 33.0 * ctas;
+      if (seg) cost += 5500;
       if (S == 1) cost += bufs == 1 ? waves * ep : ep;
-      else cost += 250.0 * S + 13.0 * MT * N + ep / S;
+      else cost += 260.0 * S + 21.0 * MT * N + 0.2 * ep / S + 10500.0 * (rounds - 1);
       if (best_cost < 0 || cost < best_cost) {
         best_cost = cost;
-        best = PairPlan{N, nt, m_tiles, KBT, S, stages, bufs, seg, planes, clusters * 2 * S,
+        best = PairPlan{N, nt, m_tiles, KBT, S, stages, bufs, seg, planes, rounds, clusters * 2 * S,
                         (size_t)stages * stage + 1024};
       }
     }
