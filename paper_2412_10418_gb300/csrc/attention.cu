@@ -16,8 +16,8 @@
 //
 // Score loop: a warp owns QPW (2, 4 or 5) query vectors (broadcast reads), its lanes own keys lane
 // and lane + 32 (rows of 132 floats: conflict-free 128-bit reads). Output loop: lanes own 4
-// (or 2) consecutive dims of the warp's query vectors, reading P by broadcast and V
-// row-contiguously. All 8 warps have query vectors: a query block is 8 * QPW of them.
+// (or 2) consecutive dims of the warp's query vectors, reading P by broadcast (four keys at a time) and
+// V row-contiguously. All 8 warps have query vectors: a query block is 8 * QPW of them.
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -43,8 +43,8 @@ int g_max_cluster = 8;               // 16 where non-portable clusters of this k
 template <int HD>
 struct AttnSmem {
   static constexpr int QP = HD + 4;        // padded row pitch of Q and K
-  static constexpr int PP = AQB + 4;       // row pitch of P (4-way store conflicts at most)
-  static constexpr size_t floats = (size_t)AQB * QP + (size_t)ACH * QP + (size_t)ACH * HD + (size_t)ACH * PP;
+  static constexpr int PP = ACH + 4;       // row pitch of P
+  static constexpr size_t floats = (size_t)AQB * QP + (size_t)ACH * QP + (size_t)ACH * HD + (size_t)AQB * PP;
   static constexpr size_t bytes = floats * sizeof(float);
 };
 
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(ATHREADS, 2) k_attn(AttnArgs a) {
   float* qS = reinterpret_cast<float*>(sm4);   // [QB][QP]  pre-scaled queries
   float* kS = qS + AQB * SL::QP;                 // [ACH][QP]; after the chunks: partial o [QB][HD]
   float* vS = kS + ACH * SL::QP;                 // [ACH][HD]
-  float* pS = vS + ACH * HD;                    // [ACH][PP] probabilities
+  float* pS = vS + ACH * HD;                    // [QB][PP] probabilities
   __shared__ attn::Layout<QB> L;
   __shared__ int s_nkeys;
   __shared__ float s_pm[QB], s_pl[QB];          // the block's partial (m, l) per query vector
@@ -226,50 +226,40 @@ __global__ void __launch_bounds__(ATHREADS, 2) k_attn(AttnArgs a) {
 #pragma unroll
       for (int c2 = 0; c2 < DPL; ++c2) o[q][c2] *= alpha[q];
     }
-    if constexpr (QPW == 4) {
-      *reinterpret_cast<float4*>(pS + lane * SL::PP + q0) = make_float4(p0[0], p0[1], p0[2], p0[3]);
-      *reinterpret_cast<float4*>(pS + (lane + 32) * SL::PP + q0) =
-          make_float4(p1[0], p1[1], p1[2], p1[3]);
-    } else if constexpr (QPW == 2) {
-      *reinterpret_cast<float2*>(pS + lane * SL::PP + q0) = make_float2(p0[0], p0[1]);
-      *reinterpret_cast<float2*>(pS + (lane + 32) * SL::PP + q0) = make_float2(p1[0], p1[1]);
-    } else {
 #pragma unroll
-      for (int q = 0; q < QPW; ++q) {
-        pS[lane * SL::PP + q0 + q] = p0[q];
-        pS[(lane + 32) * SL::PP + q0 + q] = p1[q];
-      }
+    for (int q = 0; q < QPW; ++q) {
+      pS[(q0 + q) * SL::PP + lane] = p0[q];
+      pS[(q0 + q) * SL::PP + lane + 32] = p1[q];
     }
     __syncwarp();
 
-    // ---- o += P V: lane -> dims [DPL*lane, DPL*lane + DPL)
-#pragma unroll 4
-    for (int t = 0; t < ACH; ++t) {
-      float pp[QPW];
-      if constexpr (QPW == 4) {
-        const float4 p4 = *reinterpret_cast<const float4*>(pS + t * SL::PP + q0);
-        pp[0] = p4.x; pp[1] = p4.y; pp[2] = p4.z; pp[3] = p4.w;
-      } else if constexpr (QPW == 2) {
-        const float2 p2 = *reinterpret_cast<const float2*>(pS + t * SL::PP + q0);
-        pp[0] = p2.x; pp[1] = p2.y;
-      } else {
+    // ---- o += P V: lane -> dims [DPL*lane, DPL*lane + DPL). P is read four keys at a time: one
+    //      128-bit broadcast per query vector, where a key's five scalars cost five reads
+#pragma unroll 2
+    for (int t = 0; t < ACH; t += 4) {
+      float pp[QPW][4];
 #pragma unroll
-        for (int q = 0; q < QPW; ++q) pp[q] = pS[t * SL::PP + q0 + q];
-      }
-      float v[DPL];
-      if constexpr (DPL == 4) {
-        const float4 v4 = *reinterpret_cast<const float4*>(vS + t * HD + 4 * lane);
-        v[0] = v4.x; v[1] = v4.y; v[2] = v4.z; v[3] = v4.w;
-      } else {
-        const float2 v2 = *reinterpret_cast<const float2*>(vS + t * HD + 2 * lane);
-        v[0] = v2.x; v[1] = v2.y;
+      for (int q = 0; q < QPW; ++q) {
+        const float4 p4 = *reinterpret_cast<const float4*>(pS + (q0 + q) * SL::PP + t);
+        pp[q][0] = p4.x; pp[q][1] = p4.y; pp[q][2] = p4.z; pp[q][3] = p4.w;
       }
 #pragma unroll
-      for (int q = 0; q < QPW; ++q)
+      for (int u = 0; u < 4; ++u) {
+        float v[DPL];
+        if constexpr (DPL == 4) {
+          const float4 v4 = *reinterpret_cast<const float4*>(vS + (t + u) * HD + 4 * lane);
+          v[0] = v4.x; v[1] = v4.y; v[2] = v4.z; v[3] = v4.w;
+        } else {
+          const float2 v2 = *reinterpret_cast<const float2*>(vS + (t + u) * HD + 2 * lane);
+          v[0] = v2.x; v[1] = v2.y;
+        }
 #pragma unroll
-        for (int c2 = 0; c2 < DPL; ++c2) o[q][c2] = fmaf(pp[q], v[c2], o[q][c2]);
+        for (int q = 0; q < QPW; ++q)
+#pragma unroll
+          for (int c2 = 0; c2 < DPL; ++c2) o[q][c2] = fmaf(pp[q][u], v[c2], o[q][c2]);
+      }
     }
-    __syncwarp();   // pS columns of this warp are rewritten by its next chunk
+    __syncwarp();   // pS rows of this warp are rewritten by its next chunk
   }
 
   // ---- the block's partial (m, l, o) per query vector into shared memory (o over kS)
