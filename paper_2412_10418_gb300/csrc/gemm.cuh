@@ -134,6 +134,145 @@ __device__ __forceinline__ void qkv_rows(const GemmArgs& a, int r0, int n, QkvRo
 
 __device__ __forceinline__ float silu_f(float g) { return g / (1.0f + expf(-g)); }
 
+// Sum v[i] over the warp's lanes for all i; lane l then holds the sum of index l * NR / 32 in
+// v[0] (NR a power of two up to 16: a transposing butterfly, NR shuffles and a few instead of 5 NR).
+template <int NR>
+__device__ __forceinline__ void warp_sums(float (&v)[NR]) {
+  int n = NR;
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) {
+    if (n > 1) {
+      const bool upper = (threadIdx.x & off) != 0;
+#pragma unroll
+      for (int i = 0; i < NR / 2; ++i) {
+        if (i < n / 2) {
+          const float send = upper ? v[i] : v[i + n / 2];
+          const float keep = upper ? v[i + n / 2] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+      }
+      n >>= 1;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    }
+  }
+}
+
+// Epilogue on registers: finish NR activation rows row0 .. row0 + NR - 1 (the first `rows` of them)
+// of one output per lane. STORE / RESID: L is the weight row, y0 its sums. SWIGLU: the feature, y0
+// its gate and y1 its up sums. QKV: the pair (head, e) = (L / (hd / 2), L % (hd / 2)) over the
+// stacked heads, y0 and y1 the sums of dims e and e + hd / 2. rs: row scales of row0 on (a.in_ss),
+// qr: QKV row destinations of row0 on. Whole warps call it with 32 consecutive L from a multiple
+// of 32; row0 and rows are warp-uniform.
+template <int MODE, int NR>
+__device__ __forceinline__ void finish_rows(const GemmArgs& a, int L, int row0, int rows,
+                                            const float (&y0)[NR], const float (&y1)[NR],
+                                            const float* rs, const QkvRow* qr) {
+  using T = __nv_bfloat16;
+  const int lane = threadIdx.x & 31;
+  const bool scaled = a.in_ss != nullptr;
+  if constexpr (MODE == EPI_STORE) {
+    const int n = L;
+    float* const out = a.out_f32 + (size_t)row0 * a.ld_out + n;
+    const size_t ld = a.ld_out;
+    if (n >= a.n_virtual) return;
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+      if (i < rows) out[i * ld] = scaled ? y0[i] * rs[i] : y0[i];
+  } else if constexpr (MODE == EPI_RESID) {
+    const int n = L;
+    if (n >= a.n_virtual) return;   // warp-uniform: n_virtual = d_model, a multiple of 64
+    const size_t ld = a.ld_out, plane = (size_t)a.act_plane;
+    float* const out = a.out_f32 + (size_t)row0 * ld + n;
+    T* const nx = reinterpret_cast<T*>(a.next_x);
+    T* const nxr = nx + (size_t)row0 * ld + n;
+    float h[NR];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) h[i] = i < rows ? out[i * ld] : 0.f;
+    const float g = nx ? to_f32<T>(reinterpret_cast<const T*>(a.next_g)[n]) : 0.f;
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      if (i < rows) {
+        h[i] += scaled ? y0[i] * rs[i] : y0[i];
+        out[i * ld] = h[i];
+        if (nx) store_act<T>(nxr, plane, i * ld, h[i] * g);
+      }
+    }
+    if (a.out_ss) {
+      const int i = lane * NR / 32;
+      const bool writer = lane % (32 / NR) == 0 && i < rows;
+      const size_t at = (size_t)(row0 + i) * a.ld_ss + (n >> 5);
+      float s[NR];
+#pragma unroll
+      for (int q = 0; q < NR; ++q) s[q] = h[q] * h[q];
+      warp_sums<NR>(s);
+      if (writer) a.out_ss[at] = s[0];
+      if (a.head_w) {
+        const float gw = a.head_w[n] * g;
+#pragma unroll
+        for (int q = 0; q < NR; ++q) s[q] = gw * h[q];
+        warp_sums<NR>(s);
+        if (writer) a.out_hw[at] = s[0];
+      }
+    }
+  } else if constexpr (MODE == EPI_SWIGLU) {
+    const int f = L;
+    if (f >= a.d_ffn) return;
+    const size_t ld = a.ld_act, plane = (size_t)a.act_plane;
+    T* const out = reinterpret_cast<T*>(a.out_act) + (size_t)row0 * ld + f;
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      if (i < rows) {
+        const float sc = scaled ? rs[i] : 1.f;
+        store_act<T>(out, plane, i * ld, silu_f(y0[i] * sc) * (y1[i] * sc));
+      }
+    }
+  } else {   // EPI_QKV: dims e and e + hd / 2 of one head
+    const KvStore& kv = a.kv;
+    const int hd = kv.hd, half = hd >> 1, H = a.n_heads, KVH = kv.kvh;
+    const int head = L / half, e = L % half;
+    if (head >= H + 2 * KVH) return;   // warp-uniform: half is 32 or 64
+    if (head < H + KVH) {
+      float2 cs[NR];
+#pragma unroll
+      for (int i = 0; i < NR; ++i)
+        cs[i] = i < rows ? a.rope[(size_t)qr[i].pos * half + e] : make_float2(1.f, 0.f);
+      const int nq = H * hd;
+      float* const q = a.q_out + (size_t)row0 * nq + head * hd + e;
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        if (i >= rows) continue;
+        const float sc = scaled ? rs[i] : 1.f;
+        const float u = y0[i] * sc, v = y1[i] * sc;
+        const float ru = u * cs[i].x - v * cs[i].y, rv = v * cs[i].x + u * cs[i].y;
+        if (head < H) {
+          q[(size_t)i * nq] = ru;
+          q[(size_t)i * nq + half] = rv;
+        } else if (qr[i].where) {
+          float* const d = qr[i].where == 1
+                               ? kv.pool + qr[i].base + ((size_t)(head - H) * hd << kv.page_shift)
+                               : kv.tail + qr[i].base + (size_t)(head - H) * hd;
+          d[e] = ru;
+          d[e + half] = rv;
+        }
+      }
+    } else {
+      const int vh = head - H - KVH;
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        if (i >= rows || !qr[i].where) continue;
+        const float sc = scaled ? rs[i] : 1.f;
+        float* const d =
+            qr[i].where == 1
+                ? kv.pool + qr[i].base + ((size_t)(KVH + vh) * hd << kv.page_shift)
+                : kv.tail + qr[i].base + ((size_t)kv.n_tail_slots * KVH + vh) * hd;
+        d[e] = y0[i] * sc;
+        d[e + half] = y1[i] * sc;
+      }
+    }
+  }
+}
+
 // Apply the epilogue to a finished fp32 tile: tile[r * ldt + v] holds y for activation row
 // r0 + r and virtual row v0 + v (v in [0, 128)), for r in [0, rt). s_rs[r] is the input row
 // scale of row r0 + r when a.in_ss is set (see input_row_scales). Run by `nthr` threads (a

@@ -75,143 +75,6 @@ __host__ __device__ __forceinline__ uint32_t pow2_cols(int n) {
   return c;
 }
 
-// Sum v[i] over the warp's lanes for all i; lane l then holds the sum of index l * NR / 32 in
-// v[0] (NR 8 or 16: a transposing butterfly, NR shuffles and a few instead of 5 NR).
-template <int NR>
-__device__ __forceinline__ void warp_sums(float (&v)[NR]) {
-  int n = NR;
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    if (n > 1) {
-      const bool upper = (threadIdx.x & off) != 0;
-#pragma unroll
-      for (int i = 0; i < NR / 2; ++i) {
-        if (i < n / 2) {
-          const float send = upper ? v[i] : v[i + n / 2];
-          const float keep = upper ? v[i + n / 2] : v[i];
-          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-      }
-      n >>= 1;
-    } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
-    }
-  }
-}
-
-// Finish NR activation rows row0 .. row0 + NR - 1 of one weight row per lane. L: the lane's
-// row in the pair's tile (0..255), tm: the tile. y0 / y1: the accumulators' sums. rs: row
-// scales of row0 on (a.in_ss), qr: QKV row destinations of row0 on. Whole warps call it; row0
-// and the bounds on rows are warp-uniform, and so is n < n_virtual in groups of 32 features.
-template <int MODE, int NR>
-__device__ __forceinline__ void finish_rows(const GemmArgs& a, int tm, int L, int row0, int rows,
-                                            const float (&y0)[NR], const float (&y1)[NR],
-                                            const float* rs, const QkvRow* qr) {
-  using T = __nv_bfloat16;
-  const int lane = threadIdx.x & 31;
-  const bool scaled = a.in_ss != nullptr;
-  if constexpr (MODE == EPI_STORE) {
-    const int n = tm * 256 + L;
-    float* const out = a.out_f32 + (size_t)row0 * a.ld_out + n;
-    const size_t ld = a.ld_out;
-    if (n >= a.n_virtual) return;
-#pragma unroll
-    for (int i = 0; i < NR; ++i)
-      if (i < rows) out[i * ld] = scaled ? y0[i] * rs[i] : y0[i];
-  } else if constexpr (MODE == EPI_RESID) {
-    const int n = tm * 256 + L;
-    if (n >= a.n_virtual) return;   // warp-uniform: n_virtual = d_model, a multiple of 64
-    const size_t ld = a.ld_out, plane = (size_t)a.act_plane;
-    float* const out = a.out_f32 + (size_t)row0 * ld + n;
-    T* const nx = reinterpret_cast<T*>(a.next_x);
-    T* const nxr = nx + (size_t)row0 * ld + n;
-    float h[NR];
-#pragma unroll
-    for (int i = 0; i < NR; ++i) h[i] = i < rows ? out[i * ld] : 0.f;
-    const float g = nx ? to_f32<T>(reinterpret_cast<const T*>(a.next_g)[n]) : 0.f;
-#pragma unroll
-    for (int i = 0; i < NR; ++i) {
-      if (i < rows) {
-        h[i] += scaled ? y0[i] * rs[i] : y0[i];
-        out[i * ld] = h[i];
-        if (nx) store_act<T>(nxr, plane, i * ld, h[i] * g);
-      }
-    }
-    if (a.out_ss) {
-      const int i = lane * NR / 32;
-      const bool writer = lane % (32 / NR) == 0 && i < rows;
-      const size_t at = (size_t)(row0 + i) * a.ld_ss + (n >> 5);
-      float s[NR];
-#pragma unroll
-      for (int q = 0; q < NR; ++q) s[q] = h[q] * h[q];
-      warp_sums<NR>(s);
-      if (writer) a.out_ss[at] = s[0];
-      if (a.head_w) {
-        const float gw = a.head_w[n] * g;
-#pragma unroll
-        for (int q = 0; q < NR; ++q) s[q] = gw * h[q];
-        warp_sums<NR>(s);
-        if (writer) a.out_hw[at] = s[0];
-      }
-    }
-  } else if constexpr (MODE == EPI_SWIGLU) {
-    const int f = tm * 256 + L;
-    if (f >= a.d_ffn) return;
-    const size_t ld = a.ld_act, plane = (size_t)a.act_plane;
-    T* const out = reinterpret_cast<T*>(a.out_act) + (size_t)row0 * ld + f;
-#pragma unroll
-    for (int i = 0; i < NR; ++i) {
-      if (i < rows) {
-        const float sc = scaled ? rs[i] : 1.f;
-        store_act<T>(out, plane, i * ld, silu_f(y0[i] * sc) * (y1[i] * sc));
-      }
-    }
-  } else {   // EPI_QKV: dims e and e + hd / 2 of one head
-    const KvStore& kv = a.kv;
-    const int hd = kv.hd, half = hd >> 1, H = a.n_heads, KVH = kv.kvh;
-    const int head = tm * (256 / half) + L / half, e = L % half;
-    if (head >= H + 2 * KVH) return;   // warp-uniform: half is 32 or 64
-    if (head < H + KVH) {
-      float2 cs[NR];
-#pragma unroll
-      for (int i = 0; i < NR; ++i)
-        cs[i] = i < rows ? a.rope[(size_t)qr[i].pos * half + e] : make_float2(1.f, 0.f);
-      const int nq = H * hd;
-      float* const q = a.q_out + (size_t)row0 * nq + head * hd + e;
-#pragma unroll
-      for (int i = 0; i < NR; ++i) {
-        if (i >= rows) continue;
-        const float sc = scaled ? rs[i] : 1.f;
-        const float u = y0[i] * sc, v = y1[i] * sc;
-        const float ru = u * cs[i].x - v * cs[i].y, rv = v * cs[i].x + u * cs[i].y;
-        if (head < H) {
-          q[(size_t)i * nq] = ru;
-          q[(size_t)i * nq + half] = rv;
-        } else if (qr[i].where) {
-          float* const d = qr[i].where == 1
-                               ? kv.pool + qr[i].base + ((size_t)(head - H) * hd << kv.page_shift)
-                               : kv.tail + qr[i].base + (size_t)(head - H) * hd;
-          d[e] = ru;
-          d[e + half] = rv;
-        }
-      }
-    } else {
-      const int vh = head - H - KVH;
-#pragma unroll
-      for (int i = 0; i < NR; ++i) {
-        if (i >= rows || !qr[i].where) continue;
-        const float sc = scaled ? rs[i] : 1.f;
-        float* const d =
-            qr[i].where == 1
-                ? kv.pool + qr[i].base + ((size_t)(KVH + vh) * hd << kv.page_shift)
-                : kv.tail + qr[i].base + ((size_t)kv.n_tail_slots * KVH + vh) * hd;
-        d[e] = y0[i] * sc;
-        d[e + half] = y1[i] * sc;
-      }
-    }
-  }
-}
-
 // 16 columns of an accumulator, plus those of its lo plane `lo` columns on where it has one.
 __device__ __forceinline__ void load_sums(uint32_t taddr, uint32_t lo, float (&v)[16]) {
   tc::tmem_ld16(taddr, v);
@@ -225,7 +88,7 @@ __device__ __forceinline__ void load_sums(uint32_t taddr, uint32_t lo, float (&v
 
 // finish_rows of 16 rows from c on (of the tile's `rows`, the first of which is r0), kFin at a time.
 template <int MODE>
-__device__ __forceinline__ void finish_sums(const GemmArgs& a, int tm, int L, int r0, int c,
+__device__ __forceinline__ void finish_sums(const GemmArgs& a, int L, int r0, int c,
                                             int rows, const float (&v0)[16],
                                             const float (&v1)[16], const float* rs,
                                             const QkvRow* qr) {
@@ -238,7 +101,7 @@ __device__ __forceinline__ void finish_sums(const GemmArgs& a, int tm, int L, in
       y0[i] = v0[h + i];
       y1[i] = v1[h + i];
     }
-    finish_rows<MODE, kFin>(a, tm, L, r0 + c + h, rows - c - h, y0, y1, rs + c + h,
+    finish_rows<MODE, kFin>(a, L, r0 + c + h, rows - c - h, y0, y1, rs + c + h,
                             qr + (MODE == EPI_QKV ? c + h : 0));
   }
 }
@@ -453,7 +316,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             float y0[16], y1[16];
             load_sums(d + c, lo, y0);
             if constexpr (MT == 2) load_sums(d + N + c, lo, y1);
-            finish_sums<MODE>(a, tm, L, r0, c, rows, y0, MT == 2 ? y1 : y0, s_rs, s_qkv);
+            finish_sums<MODE>(a, tm * 256 + L, r0, c, rows, y0, MT == 2 ? y1 : y0, s_rs, s_qkv);
           }
         }   // (split K: below, straight from TMEM)
         tc::tc_fence_before();
@@ -499,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int j = 0; j < kChunks; j += MT) {
             const int c = 16 * (cg + kGroups * (j / MT));
             if (c < rows)
-              finish_sums<MODE>(a, tm, L, r0, c, rows, acc[j], acc[j + MT - 1], s_rs, s_qkv);
+              finish_sums<MODE>(a, tm * 256 + L, r0, c, rows, acc[j], acc[j + MT - 1], s_rs, s_qkv);
           }
         } else {
 #pragma unroll
@@ -563,7 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if constexpr (MT == 2) y1[i] += tc::ld_cluster_f32(src + NH * 512 + ci);
           }
         }
-        finish_rows<MODE, 8>(a, tm, L, r0 + b0 + c, min(8, rb - c), y0, y1, s_rs + b0 + c,
+        finish_rows<MODE, 8>(a, tm * 256 + L, r0 + b0 + c, min(8, rb - c), y0, y1, s_rs + b0 + c,
                              s_qkv + (MODE == EPI_QKV ? b0 + c : 0));
       }
     }

@@ -79,6 +79,9 @@ __device__ __forceinline__ int unit_owner(int u, int U, int C) { return ((u + 1)
 constexpr int kMaxContrib = 256;   // contributors to one tile (bounded on the host)
 constexpr int kMaxSplit = 8;       // target blocks per tile when tiles are few
 
+// kRegs: the cluster split-K finishes its rows on registers (QKV and residual projections with
+// enough rows per block: launch_gemm_tc).
+template <bool kRegs>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_tc(const __grid_constant__ TcMaps maps, const __grid_constant__ GemmArgs a, TcPlan p,
               float* part, int* tile_cnt) {
@@ -93,6 +96,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ int s_abort, s_last;
   __shared__ int s_slot_off[kMaxContrib];   // reducer: scratch offset (floats) per contributor
   __shared__ float s_rs[kPairRows];          // input row scales (RMSNorm folded into the GEMM)
+  __shared__ QkvRow s_qkv[kRegs ? kPairRows : 1];   // QKV: where this block's rows go
 
   uint8_t* smem = smem_raw + ((1024 - (tc::smem_u32(smem_raw) & 1023)) & 1023);
   const int NP = p.n_pad, S = p.stages, KBT = p.kb_total;
@@ -167,6 +171,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   pdl_launch_dependents();
   const uint32_t tmem = tmem_base;
 
+  bool gave_up = true;   // (epilogue warps: false once every accumulator has been drained)
   if (warp == 0) {
     if (lane == 0) {
       // ---------------- TMA producer
@@ -247,7 +252,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     int seg = 0;
     int u = u0;
     const int R = min(a.R, NP);
-    if (a.in_ss) {   // once per block, while the first accumulator fills
+    if constexpr (kRegs) {   // what this block's rows need, while the accumulator fills
+      const int ra = (c % SK) * R / SK, rb = (c % SK + 1) * R / SK;
+      if (a.in_ss) input_row_scales(a, ra, rb - ra, s_rs, etid, kEpThreads);
+      if (a.mode == EPI_QKV) qkv_rows(a, ra, rb - ra, s_qkv, etid, kEpThreads);
+      tc::named_barrier(1, kEpThreads);
+    } else if (a.in_ss) {   // once per block
       input_row_scales(a, 0, R, s_rs, etid, kEpThreads);
       tc::named_barrier(1, kEpThreads);
     }
@@ -270,19 +280,22 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int r0 = 0; r0 < NP; r0 += kEpRows) {
         const int rows = min(kEpRows, NP - r0);
         for (int c0 = 0; c0 < rows; c0 += 16) {
-          float v[16], w[16];
-          tc::tmem_ld16(d + (uint32_t)(r0 + c0), v);
-          tc::tmem_ld16(d + (uint32_t)(NP + r0 + c0), w);
+          uint32_t v[16], w[16];
+          tc::tmem_ld16_nowait(d + (uint32_t)(r0 + c0), v);
+          tc::tmem_ld16_nowait(d + (uint32_t)(NP + r0 + c0), w);
+          tc::tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] += w[i];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) tileS[(c0 + i) * kTileLd + quarter * 32 + lane] = v[i];
+          for (int i = 0; i < 16; ++i)
+            tileS[(c0 + i) * kTileLd + quarter * 32 + lane] =
+                __uint_as_float(v[i]) + __uint_as_float(w[i]);
         }
+        // cluster split-K: the partial stays in tileS (ep_rows == NP: one chunk) until the
+        // cluster reduction at the end, whose barrier publishes it
+        if (kRegs) continue;
         tc::named_barrier(1, kEpThreads);
         const int rt = max(0, min(rows, R - r0));
         if (SK > 0) {
-          // cluster split-K: the partial stays in tileS (ep_rows == NP: one chunk) until the
-          // cluster reduction at the end
+          // (summed and finished at the end)
         } else if (whole) {
           tile_epilogue<__nv_bfloat16>(a, t * 128, r0, rt, tileS, kTileLd, s_rs + r0, etid,
                                        kEpThreads);
@@ -296,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       tc::tc_fence_before();
       tc::mbar_arrive(&acce_bar[acc]);   // accumulator drained: the MMA lane may reuse it
-      if (!whole && SK == 0) {
+      if (!kRegs && !whole && SK == 0) {
         const int cf = unit_owner(t * KBT, U, C);
         const int cl = unit_owner((t + 1) * KBT - 1, U, C);
         // publish this block's partial and count it (one acquire-release atomic after the
@@ -338,8 +351,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               *reinterpret_cast<float4*>(tileS + (i >> 5) * kTileLd + (i & 31) * 4) = sum;
             }
             tc::named_barrier(1, kEpThreads);
-            tile_epilogue<__nv_bfloat16>(a, t * 128, r0, rt, tileS, kTileLd, s_rs + r0,
-                                                etid, kEpThreads);
+            tile_epilogue<__nv_bfloat16>(a, t * 128, r0, rt, tileS, kTileLd, s_rs + r0, etid,
+                                         kEpThreads);
             tc::named_barrier(1, kEpThreads);
           }
           if (etid == 0) tile_cnt[t] = 0;
@@ -348,17 +361,92 @@ __global__ void __launch_bounds__(kThreads, 1)
       u = seg_end;
       ++seg;
     }
+    gave_up = u < u1;
   }
-  if (SK > 0) {
+  if constexpr (kRegs) {
     // ---- cluster split-K reduction: rank r sums rows [r*R/SK, (r+1)*R/SK) of the SK partial
+    //      tiles in rank order (distributed shared memory) and finishes them on registers: a lane
+    //      is one output, in QKV both values of a RoPE pair. (Through a summed tile in shared
+    //      memory and tile_epilogue it cost two more barriers and, in QKV, the rows' descriptors
+    //      and pages after the sums.)
+    tc::cluster_arrive();               // this block's partial tile is complete (release)
+    tc::cluster_wait();                 // every block's is (acquire)
+    // the closing barrier is met as soon as a warp's last sums are read: its second phase runs
+    // while the epilogue writes
+    bool arrived = false;
+    if (warp >= 2 && !gave_up) {
+      const int R = min(a.R, NP), r = c % SK, t = c / SK, w = warp & 3;
+      const int ra = r * R / SK, rb = (r + 1) * R / SK;
+      const uint32_t tile_s = tc::smem_u32(tileS);
+      // sums of rows row .. row + NR - 1 of the share at tile columns v0 and v1, eight blocks'
+      // loads in flight per row
+      auto sums = [&](int row, int v0, int v1, auto& y0, auto& y1) {
+        constexpr int NR = sizeof(y0) / sizeof(float);
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+          y0[i] = y1[i] = 0.f;
+          if (row + i >= rb) continue;   // warp-uniform
+          const uint32_t at = tile_s + (uint32_t)((row + i) * kTileLd) * 4;
+          for (int q0 = 0; q0 < SK; q0 += 8) {
+            float a0[8], a1[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              if (q0 + q >= SK) break;
+              const uint32_t src = tc::map_cluster_rank(at, (uint32_t)(q0 + q));
+              a0[q] = tc::ld_cluster_f32(src + v0 * 4);
+              if (v1 >= 0) a1[q] = tc::ld_cluster_f32(src + v1 * 4);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              if (q0 + q >= SK) break;
+              y0[i] += a0[q];
+              if (v1 >= 0) y1[i] += a1[q];
+            }
+          }
+        }
+      };
+      if (a.mode == EPI_RESID) {   // warp w: features 32 w ..
+        for (int row = ra; row < rb; row += 4) {
+          float y0[4], y1[4];
+          sums(row, w * 32 + lane, -1, y0, y1);
+          if (row + 4 >= rb) {
+            tc::cluster_arrive();
+            arrived = true;
+          }
+          finish_rows<EPI_RESID, 4>(a, t * 128 + w * 32 + lane, row, rb - row, y0, y1,
+                                    s_rs + row - ra, s_qkv);
+        }
+      } else {   // QKV: warps w and w + 2 share 32 of the tile's 64 pairs, rows two by two
+        const int pi = (w & 1) * 32 + lane;
+        int v0 = pi, v1 = pi + 64;
+        if (a.kv.hd == 64) {   // two heads of 32 pairs per tile
+          v0 = pi + (pi & 32);
+          v1 = v0 + 32;
+        }
+        for (int row = ra + (w >> 1) * 2; row < rb; row += 4) {
+          float y0[2], y1[2];
+          sums(row, v0, v1, y0, y1);
+          if (row + 4 >= rb) {
+            tc::cluster_arrive();
+            arrived = true;
+          }
+          finish_rows<EPI_QKV, 2>(a, t * 64 + pi, row, rb - row, y0, y1, s_rs + row - ra,
+                                  s_qkv + row - ra);
+        }
+      }
+    }
+    if (!arrived) tc::cluster_arrive();
+    tc::cluster_wait();                 // no block leaves while its tile may still be read
+  } else if (SK > 0) {
+    // ---- the same with few rows per block: rank r sums rows [r*R/SK, (r+1)*R/SK) of the SK partial
     //      tiles in rank order (distributed shared memory) into a free pipeline stage and runs
     //      the epilogue on them
     // the epilogue warps agree on whether the block gave up (the two named barriers below
     // must be reached by all of them or by none)
-    const bool gave_up = warp >= 2 ? tc::named_barrier_or(1, kEpThreads, s_abort != 0) : true;
+    const bool none = warp >= 2 ? tc::named_barrier_or(1, kEpThreads, s_abort != 0) : true;
     tc::cluster_arrive();               // this block's partial tile is complete (release)
     tc::cluster_wait();                 // every block's is (acquire)
-    const bool reduce = warp >= 2 && !gave_up;
+    const bool reduce = warp >= 2 && !none;
     const int R = min(a.R, NP), r = c % SK, t = c / SK;
     const int ra = r * R / SK, rb = (r + 1) * R / SK;
     float* red = reinterpret_cast<float*>(smem);   // stage 0 (idle): [rb - ra][kTileLd]
@@ -507,26 +595,35 @@ int encode_bf16_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t o
 }
 
 int configure_gemm_tc() {
-  auto kernel = k_gemm_tc;
+  auto kernel = k_gemm_tc<true>;   // (the larger static part)
   cudaFuncAttributes fa;
   if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return -1;
   g_static_smem = fa.sharedSizeBytes;
-  const bool nonportable =
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-      cudaSuccess;
-  cudaGetLastError();
-  g_max_cluster = nonportable ? 16 : 8;
   // plans use at most 220 KB + 1 KB of alignment slack; a block has at most 227 KB in all
   const int dyn = (int)std::min<size_t>(220 * 1024 + 1024, 227 * 1024 - fa.sharedSizeBytes);
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) ==
-                 cudaSuccess
-             ? 0
-             : -1;
+  bool nonportable = true;
+  int rc = 0;
+  for (auto k : {k_gemm_tc<false>, k_gemm_tc<true>}) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+      nonportable = false;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
+      rc = -1;
+  }
+  cudaGetLastError();
+  g_max_cluster = nonportable ? 16 : 8;
+  return rc;
 }
 
 void launch_gemm_tc(const TcMaps& maps, const GemmArgs& a, const TcPlan& p, float* part,
                     int* tile_cnt, cudaStream_t s) {
-  auto kernel = k_gemm_tc;
+  // A cluster's rows are finished on registers where each of its blocks has enough of them: three
+  // for QKV (7B verify pass, 20 rows over 5 blocks: 14.8 -> 13.9 us; at two rows, each a round trip
+  // of 4-byte remote loads, the small model's requests lose 1.3 %), two for the residual projections
+  // (O 11.7 -> 11.1, down 20.2 -> 19.5; the draft's 4 rows over 12 blocks lose: O 4.9 -> 5.6).
+  // Gate/up keeps the tile (16 rows over 3 blocks lose 1.5 us a launch).
+  const bool regs = p.cluster && ((a.mode == EPI_QKV && a.R >= 3 * p.cluster) ||
+                                  (a.mode == EPI_RESID && a.R >= 2 * p.cluster));
+  auto kernel = regs ? k_gemm_tc<true> : k_gemm_tc<false>;
   if (p.cluster)
     launch_pdl_cluster(kernel, dim3(p.ctas), dim3(kThreads), p.smem, p.cluster, s, maps, a, p,
                        part, tile_cnt);

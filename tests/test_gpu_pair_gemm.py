@@ -36,6 +36,18 @@ def test_verify_rows_at_tile_edges(shape, batch, k, d):
     run_parity(make_setup(wl), steps=2, tol=TOL, tol_r=TOL)
 
 
+@pytest.mark.parametrize("shape", [HD64, HD128], ids=["hd64", "hd128"])
+@pytest.mark.parametrize("batch,k,d", [(1, 15, 1), (1, 12, 2), (1, 16, 3)],
+                         ids=["30rows", "36rows", "64rows"])
+def test_cluster_rows_finished_on_registers(shape, batch, k, d):
+    """At most 64 rows, enough of them per block of a cluster that QKV and the residual projections
+    are finished on registers: shares of two to eight rows, uneven ones, both head sizes."""
+    wl = synth.scaled(synth.TINY, dtype=synth.DTYPE_BF16, target=shape,
+                      draft=synth.ModelShape(vocab=shape.vocab, **DRAFT), batch=batch, k=k, d=d,
+                      prompt_len=9, max_new=8, reward_head=True)
+    run_parity(make_setup(wl), steps=2, tol=TOL, tol_r=TOL)
+
+
 @pytest.mark.parametrize("max_chunk", [0, 65, 300])
 def test_prefill_passes_above_256_rows(max_chunk):
     """Ragged prompts of 523 tokens in all, in passes of the default size, of 65 rows (remainder
