@@ -48,6 +48,17 @@ def test_cluster_rows_finished_on_registers(shape, batch, k, d):
     run_parity(make_setup(wl), steps=2, tol=TOL, tol_r=TOL)
 
 
+@pytest.mark.parametrize("shape", [HD64, HD128], ids=["hd64", "hd128"])
+@pytest.mark.parametrize("prompt_len", [952, 1016], ids=["16chunks", "17chunks"])
+def test_verify_attention_with_a_block_per_chunk_and_past_it(shape, prompt_len):
+    """65 verify rows whose 64-key chunks just fit one cluster (a chunk per block, one group of
+    warps) and are one too many for it (blocks with two chunks, two groups)."""
+    wl = synth.scaled(synth.TINY, dtype=synth.DTYPE_BF16, target=shape,
+                      draft=synth.ModelShape(vocab=shape.vocab, **DRAFT), batch=1, k=13, d=4,
+                      prompt_len=prompt_len, max_new=8, reward_head=True)
+    run_parity(make_setup(wl), steps=2, tol=TOL, tol_r=TOL)
+
+
 @pytest.mark.parametrize("max_chunk", [0, 65, 300])
 def test_prefill_passes_above_256_rows(max_chunk):
     """Ragged prompts of 523 tokens in all, in passes of the default size, of 65 rows (remainder
