@@ -483,7 +483,9 @@ PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt
   PairPlan best{};
   double best_cost = -1;
   const int nt_min = (R + kNMax - 1) / kNMax;
-  for (int nt = nt_min; nt <= nt_min + 7; ++nt) {
+  // (tiles of 128 rows are always among them: two accumulators of more rows may not be allowed)
+  const int nt_max = std::max(nt_min + 7, (R + 127) / 128);
+  for (int nt = nt_min; nt <= nt_max; ++nt) {
     if (force_nt && nt != force_nt) continue;
     const int N = ((R + nt - 1) / nt + 31) / 32 * 32;
     if (N > kNMax || (nt > nt_min && N < 32) || (nt - 1) * N >= R) continue;

@@ -68,3 +68,13 @@ def test_prefill_passes_above_256_rows(max_chunk):
                       prompt_len=260, max_new=8)
     run_parity(make_setup(wl, lens=[260, 63, 200]), steps=2, tol=TOL, tol_r=TOL,
                max_chunk=max_chunk)
+
+
+@pytest.mark.parametrize("lens", [[240] * 7 + [241], [260] * 8], ids=["1921rows", "2080rows"])
+def test_prefill_passes_of_many_row_tiles(lens):
+    """One pass of more than 15 x 128 rows: gate/up and QKV, whose two accumulators are not allowed
+    tiles of more than 128 rows here, need 16 and 17 row tiles where 256 rows would need 8 and 9."""
+    wl = synth.scaled(synth.TINY, dtype=synth.DTYPE_BF16, target=HD64,
+                      draft=synth.ModelShape(vocab=HD64.vocab, **DRAFT), batch=8, k=2, d=2,
+                      prompt_len=260, max_new=8)
+    run_parity(make_setup(wl, lens=lens), steps=1, tol=TOL, tol_r=TOL, max_chunk=4096)
