@@ -230,8 +230,8 @@ def cdsl_get_profile_launches(ctx, capacity: int = 8192):
 
 
 def cdsl_gemv_noalloc(w, x, y, stream=None):
-    """y[R, N] = x[R, K] w^T through the weight-streaming kernel with its scratch in a fixed
-    array inside the library (no device memory is allocated); see include/cdsl.h.
+    """y[R, N] = x[R, K] w^T in one weight-streaming kernel that needs no scratch in global
+    memory (no device memory is allocated); see include/cdsl.h.
 
     The C ABI sees only pointers and sizes, so the shapes, dtypes, layouts and devices are
     checked here: w bfloat16 [N, K], x float32 [R, K], y float32 [R, N], all contiguous and on

@@ -24,7 +24,8 @@
 // S, O and softmax state; their partials are added at the end. 13B verify pass (224 rows, 1,100
 // keys): 128 us per launch with one group, 112 with two, 108 with V staged by rows as K is (it
 // was transposed by 4-byte loads); 176 rows at 4,160 keys 184, 156, 144. Three planes of P and V
-// (prefill, head_dim 128) leave shared memory for one group.
+// (prefill, head_dim 128) leave shared memory for one group, and passes with a block per chunk
+// (launch_verify) have no use for a second.
 //
 // Softmax: warps w and w + 4 read TMEM lanes 32(w % 4) .. +31, so each thread owns one query
 // vector's row of scores over half the chunk's keys (the two halves exchange their row

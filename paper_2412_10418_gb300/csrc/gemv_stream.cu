@@ -1,7 +1,7 @@
 // gemv_stream.cu -- CUDA-core weight-streaming GEMM for few activation rows (R <= 8): the
-// projections of bf16 models whose K the tensor-core kernel does not take (K % 64 != 0), and
-// cdsl_gemv_noalloc. Every bf16 projection with K % 64 == 0 -- all of the synthetic workloads'
-// -- runs on the tensor-core kernel (gemm_tc.cu) instead, which streams weights faster here.
+// projections of bf16 models whose K the tensor-core kernels do not take (K % 64 != 0). Every bf16
+// projection with K % 64 == 0 -- all of the synthetic workloads' -- runs on the tensor-core
+// kernels (gemm_tc.cu, gemm_pair.cu) instead, which stream weights faster here.
 //
 // With R <= 8 rows a projection moves ~R*2 flops per weight byte: the kernel is bound by HBM
 // bandwidth on the weights. Each block owns a tile of 128 virtual output rows and one K slice

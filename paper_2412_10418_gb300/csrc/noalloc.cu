@@ -181,7 +181,7 @@ extern "C" int32_t cdsl_gemv_noalloc(const void* d_w, int32_t N, int32_t K, cons
     return CDSL_EINVAL;
   }
   if (R < 1 || R > kMaxR || K < 8 || K > kMaxK || (K % 8) || N < 1 || N > kMaxN) {
-    set_thread_error("cdsl_gemv_noalloc: sizes beyond the fixed scratch: need 1 <= R <= 8, "
+    set_thread_error("cdsl_gemv_noalloc: sizes beyond its limits: need 1 <= R <= 8, "
                      "8 <= K <= 8192 with K % 8 == 0, 1 <= N <= 32768");
     return CDSL_EINVAL;
   }
