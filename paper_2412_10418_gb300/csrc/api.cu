@@ -78,6 +78,7 @@ struct cdsl_ctx {
   int32_t* lm_dst = nullptr;
   float* gemv_part = nullptr;   // split-K partial tiles of the weight-streaming GEMM
   int32_t* gemv_cnt = nullptr;  // per-tile arrival counters
+  size_t part_floats = 0, part_tiles = 0;   // their sizes
   int plan_sms = kPlanSMs;      // SMs the tensor-core GEMM plans for: min(kPlanSMs, device's)
   int32_t* attn_zmap = nullptr; // prefill: z -> (prompt, query block)
   int attn_zmax = 0, attn_chunks = 0;
@@ -108,6 +109,7 @@ struct cdsl_ctx {
   // TMA descriptors, built on first use: (base, inner, outer, box_outer) -> map
   std::map<std::tuple<uintptr_t, int, int, int>, CUtensorMap> maps;
   int map_error = 0;
+  bool scratch_short = false;   // a projection's plan did not fit its scratch
   std::string err;
 };
 
@@ -125,6 +127,8 @@ int cuda_check(cdsl_ctx* c, const char* where) {
     return fail(c, CDSL_ECUDA, std::string(where) + ": cuTensorMapEncodeTiled failed (" +
                                    std::to_string(m) + ")");
   }
+  if (c && c->scratch_short)   // (for good: a captured step lacks the launch)
+    return fail(c, CDSL_ENOMEM, std::string(where) + ": a projection's plan exceeds its scratch");
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess)
     return fail(c, CDSL_ECUDA, std::string(where) + ": " + cudaGetErrorString(e));
@@ -288,7 +292,9 @@ size_t carve(cdsl_ctx* c, void* base) {
         part = std::max(part, (size_t)p.splits * 8 * p.tiles * 128);
         tiles = std::max(tiles, (size_t)p.tiles);
         if (c->dtype == CDSL_DTYPE_BF16 && sh[0] % 64 == 0) {
-          for (int R = 9; R <= std::min(c->R_max, kPairRows); R += 16) {  // every n_pad in use
+          // every n_pad that a pass of at most R_max rows runs at
+          const int most = (std::min(c->R_max, kPairRows) + 15) / 16 * 16;
+          for (int R = 16; R <= most; R += 16) {
             // the plan, and stream-K, which a plan falls back to where clusters do not fit
             const TcPlan t = plan_tc(sh[0], sh[1], R, kPlanSMs);
             const TcPlan sk = plan_tc(sh[0], sh[1], R, kPlanSMs, 0, 0, 0);
@@ -300,6 +306,8 @@ size_t carve(cdsl_ctx* c, void* base) {
     }
     c->gemv_part = cv.take<float>(part);
     c->gemv_cnt = cv.take<int32_t>(tiles);
+    c->part_floats = part;
+    c->part_tiles = tiles;
   }
   {  // attention: the prefill's (prompt, query block) map
     const int QB = attn_qblock();
@@ -424,6 +432,11 @@ void gemm(cdsl_ctx* c, const GemmArgs& a) {
     const TcPlan p = pair ? TcPlan{} : plan_tc(a.K, a.n_virtual, a.R, c->plan_sms);
     const PairPlan pp =
         pair ? plan_pair(a.mode, a.K, a.n_virtual, a.R, c->plan_sms) : PairPlan{};
+    // (carve() sizes both over every plan: a launch that would pass them is refused)
+    if (!pair && (tc_scratch_floats(p) > c->part_floats || (size_t)p.tiles > c->part_tiles)) {
+      c->scratch_short = true;
+      return;
+    }
     TcMaps maps;
     for (int s = 0; s < 3; ++s) {
       const int seg = s < a.n_seg ? s : 0;

@@ -139,6 +139,23 @@ def test_step1_budget_2_adds_the_round_buffers(cdsl):
     assert n2 - n1 >= tails * wl.batch
 
 
+@pytest.mark.parametrize("k,d,prompt,rows", [(1, 1, 4, 4), (4, 4, 8, 20), (4, 4, 18, 20),
+                                             (6, 5, 8, 36), (10, 4, 8, 50), (13, 4, 8, 65)])
+def test_workspace_holds_the_stream_k_partials_of_every_pass(cdsl, k, d, prompt, rows):
+    """A projection of 135 weight tiles (gate/up of d_ffn 8640: too many for clusters, too few for a
+    block per tile) runs stream-K over 304 blocks, each with two partial tiles of 128 features by the
+    pass's rows rounded up to 16. The workspace holds them for the pass with the most rows (`rows`,
+    at most 64 on this kernel) beside the three activation buffers of 32-row multiples."""
+    shape = synth.ModelShape(n_layers=1, d_model=192, n_heads=3, n_kv_heads=1, d_ffn=8640, vocab=264)
+    small = synth.ModelShape(n_layers=1, d_model=64, n_heads=1, n_kv_heads=1, d_ffn=64, vocab=264)
+    wl = synth.scaled(synth.TINY, dtype=synth.DTYPE_BF16, target=shape, draft=small, batch=1, k=k,
+                      d=d, prompt_len=prompt, max_new=4)
+    n_pad = (min(rows, 64) + 15) // 16 * 16
+    partials = 4 * 304 * 2 * n_pad * 128
+    activations = 3 * 4 * ((rows + 31) // 32 * 32) * shape.d_ffn
+    assert cdsl.cdsl_workspace_size(*cfgs(cdsl, wl)) >= partials + activations
+
+
 def test_get_step1_needs_a_context(cdsl):
     assert cdsl.lib().cdsl_get_step1(None, None, None, None) == 1   # CDSL_EINVAL
 

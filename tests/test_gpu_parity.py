@@ -349,3 +349,16 @@ def test_tiny_cdlh_appx_on_the_same_kernels():
         ref = oracle.cdlh_generate(tgt, drf, drf, s.prompts[b].tolist(), s.keywords[b].tolist(),
                                    run, s.w_head)
         assert states[b].T == ref.T
+
+
+@pytest.mark.parametrize("k,d,prompt", [(1, 1, 4), (4, 4, 8), (10, 4, 8)],
+                         ids=["4rows", "20rows", "50rows"])
+def test_stream_k_passes_of_few_rows(k, d, prompt):
+    """135 gate/up tiles run stream-K, with prompts so short that the verify pass (or a prefill of 4
+    rows) is the pass with the most rows: its partial tiles, at the row count rounded up to 16, are
+    the largest that the workspace holds."""
+    shape = synth.ModelShape(n_layers=2, d_model=192, n_heads=3, n_kv_heads=1, d_ffn=8640, vocab=264)
+    small = synth.ModelShape(n_layers=1, d_model=64, n_heads=1, n_kv_heads=1, d_ffn=64, vocab=264)
+    wl = synth.scaled(synth.TINY, dtype=synth.DTYPE_BF16, target=shape, draft=small, batch=1, k=k,
+                      d=d, prompt_len=prompt, max_new=6)
+    run_parity(make_setup(wl), steps=2, tol=1e-3, tol_r=1e-3)
