@@ -37,7 +37,7 @@
 // as the O projection's hi/lo input.
 //
 // One thread issues every MMA; tcgen05.commit arrives on an mbarrier that the consumers wait
-// on (bounded by the launch's wait limit: on expiry CDSL_ETIMEOUT is latched and the block
+// on (bounded by the launch's wait limit: on expiry CDSL_ETIMEOUT is latched and the group
 // skips its remaining chunks, waits for its own MMAs in flight and still meets every cluster
 // barrier).
 #include <algorithm>
@@ -175,6 +175,11 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
   pdl_launch_dependents();    // (this block has its TMEM before any of the next kernel's)
   const int grp = threadIdx.x / GTHREADS, tid = threadIdx.x % GTHREADS;
   auto group_sync = [&] { tc::named_barrier(1 + grp, GTHREADS); };
+  // A group gives up as one: each of its threads brings its own failure to a barrier that ORs them.
+  // (From a flag in shared memory read after a barrier, a slow warp could see what a fast one set at
+  // its next wait, and the group's warps would then wait at different barriers.)
+  bool failed = false;
+  auto group_failed = [&] { return failed = tc::named_barrier_or(1 + grp, GTHREADS, failed); };
   const uint32_t tmem = s_tmem + (uint32_t)grp * SM::T_GROUP;
   const uint32_t t_s = tmem, t_o = tmem + 64;      // columns: S [0, 64), O [64, 64 + HD)
   const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
@@ -272,7 +277,7 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
     if (!kPreV) load_v(i);
     // the group's previous P V has completed: K, V and P may be overwritten
     if (nproc > 0 && !tc::mbar_wait(&bar_o[grp], (nproc - 1) & 1, a.status, a.wait_ns))
-      s_abort[grp] = 1;
+      failed = true;
     if (i + NG < nb_chunks) kptrs(i + NG);
     // ---- stage the chunk: split the loaded K and V into hi/lo and store
 #pragma unroll
@@ -298,8 +303,7 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
       for (int n = 0; n < NP; ++n) st_shared16(smg, off + n * SM::V_PLANE, p[n]);
     }
     tc::fence_proxy_async();
-    group_sync();
-    if (s_abort[grp]) break;
+    if (group_failed()) break;
     // ---- S = Q K^T (hi.hi + hi.lo + lo.hi over the head dimension)
     if (tid == kIssuer) {
       tc::tc_fence_after();
@@ -329,7 +333,7 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
     float s[2][16];
     float mx = -INFINITY;
     if (!sok) {
-      s_abort[grp] = 1;
+      failed = true;
     } else {
       tc::tc_fence_after();
       uint32_t r[2][16];
@@ -351,8 +355,7 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
         }
       s_mx[grp][half][qi] = mx;
     }
-    group_sync();
-    if (s_abort[grp]) break;
+    if (group_failed()) break;
     mx = fmaxf(s_mx[grp][0][qi], s_mx[grp][1][qi]);   // the row's maximum, the same in both halves
     {
       // raise the reference where a row's maximum passed it by more than kLazy: its earlier
@@ -437,8 +440,8 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
   // ---- the block's partial (m, l, o) per query vector into shared memory (o over everything):
   //      each half writes its half of the row's columns; l is the sum of the halves' shares. A
   //      second group leaves its partial there for the first one to add to its own.
-  if (nproc > 0 && !tc::mbar_wait(&bar_o[grp], (nproc - 1) & 1, a.status, a.wait_ns))
-    s_abort[grp] = 1;
+  if (failed || (nproc > 0 && !tc::mbar_wait(&bar_o[grp], (nproc - 1) & 1, a.status, a.wait_ns)))
+    s_abort[grp] = 1;   // (read after the next barrier, no longer written there)
   if (half == 1) s_mx[grp][1][qi] = l_run;
   __syncthreads();
   float* const s_po = reinterpret_cast<float*>(sm);              // [TQB][OP]

@@ -107,3 +107,36 @@ def test_expired_waits_in_the_large_row_gemm_and_tensor_core_attention():
     eng2, states, rep, adopted, n = run_parity(s, steps=2, tol=2e-2, tol_r=2e-2)
     assert n == 2 and eng2.status() == cdsl.CDSL_OK
     eng2.close()
+
+
+@pytest.mark.parametrize("heads", [(5, 1, 320), (3, 3, 384)], ids=["hd64", "hd128"])
+@pytest.mark.parametrize("prompt_len", [500, 1500], ids=["one_group", "two_groups"])
+def test_expired_waits_in_attention_blocks_of_many_chunks(heads, prompt_len):
+    """65 verify rows and prefill passes on the tensor-core attention, with a block per chunk and
+    with several chunks per block (two groups of warps): at a wait limit of 0 each group's threads
+    give up together wherever in the chunk loop one of them does, so every launch ends, several
+    steps and a prefill in a row."""
+    import torch
+    import paper_2412_10418_gb300 as cdsl
+    from cdsl_parity import run_parity
+
+    H, KVH, D = heads
+    shape = synth.ModelShape(n_layers=2, d_model=D, n_heads=H, n_kv_heads=KVH, d_ffn=576, vocab=520)
+    small = synth.ModelShape(n_layers=1, d_model=128, n_heads=2, n_kv_heads=1, d_ffn=192, vocab=520)
+    s = make_setup(synth.scaled(synth.TINY, dtype=synth.DTYPE_BF16, target=shape, draft=small,
+                                batch=1, k=13, d=4, prompt_len=prompt_len, max_new=16))
+    eng = engine(s)
+    eng.step()
+    assert eng.status() == cdsl.CDSL_OK
+    cdsl.cdsl_set_wait_limit(eng.ctx, 0)
+    for _ in range(4):
+        eng.step()
+        assert eng.status() == cdsl.CDSL_ETIMEOUT
+    eng.prefill(torch.from_numpy(s.prompts), s.lens, torch.from_numpy(s.keywords))
+    assert eng.status() == cdsl.CDSL_ETIMEOUT
+    torch.cuda.synchronize()
+    eng.close()
+
+    eng2, states, rep, adopted, n = run_parity(s, steps=1, tol=1e-3, tol_r=1e-3)
+    assert n == 1 and eng2.status() == cdsl.CDSL_OK
+    eng2.close()
