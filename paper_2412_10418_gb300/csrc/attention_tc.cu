@@ -10,11 +10,19 @@
 // Per chunk, with every operand a K-major bf16 tile in 128-byte-swizzled shared memory:
 //   S = Q K^T      M = 128 query vectors, N = 64 keys, K = head_dim  -> TMEM columns [0, 64)
 //   O += P V       M = 128 query vectors, N = head_dim, K = 64 keys   -> TMEM columns [64, ..)
-// fp32 accuracy from bf16 operands: every fp32 input x is split into hi = bf16(x) and
-// lo = bf16(x - hi), and each product is hi.hi + hi.lo + lo.hi (lo.lo, about 2^-18 of the
-// product, is dropped), accumulated in fp32. The K/V cache stays fp32 in HBM; the block
-// converts each chunk while staging it (rows of keys: the score product's K-major B operand, and
-// the P V product's MN-major one). Staging is software-pipelined: the next chunk's K rows are
+//                  (three planes: O = P V, added up in registers)
+// fp32 inputs from bf16 operands: every fp32 input x is split into planes. Verify passes take two,
+// hi = bf16(x) and lo = bf16(x - hi), and each product is hi.hi + hi.lo + lo.hi (lo.lo, about 2^-18
+// of the product, is dropped). Prefill passes, whose K/V cache carries every later step and which
+// otherwise run in fp32 on the CUDA cores, take three (x to 2^-25) and the six products down to
+// lo.hi. Every MMA truncates the sum that it adds to: the small products therefore go first, and in a prefill pass a chunk's P V
+// starts anew and is added to fp32 sums in registers, rounded to nearest. Output of 1024 rows at
+// 3072 to 4096 keys, against 64 bits: 2.5e-6 of its norm, as of the CUDA-core kernel (nearly all of
+// it the rounding of the output to hi and lo planes); with Q and K in two planes and one chain over
+// the chunks 9.8e-6, and 2.7e-5 at scores of standard deviation 25 (2.6e-6, CUDA cores 3.2e-6). It
+// costs a tenth of the launch: 792 -> 891 us (CUDA cores 2235). The K/V cache stays fp32 in HBM; the
+// block converts each chunk while staging it (rows of keys: the score product's K-major B operand,
+// and the P V product's MN-major one). Staging is software-pipelined: the next chunk's K rows are
 // loaded into registers while this chunk's softmax runs and stored once its P V has completed. Q
 // is split once per block, pre-scaled by log2(e) / sqrt(head_dim) (scores in base 2).
 //
@@ -23,15 +31,15 @@
 // alternate chunks of the block, each with its own K, V and P in shared memory (P over K) and its own
 // S, O and softmax state; their partials are added at the end. 13B verify pass (224 rows, 1,100
 // keys): 128 us per launch with one group, 112 with two, 108 with V staged by rows as K is (it
-// was transposed by 4-byte loads); 176 rows at 4,160 keys 184, 156, 144. Three planes of P and V
-// (prefill, head_dim 128) leave shared memory for one group, and passes with a block per chunk
+// was transposed by 4-byte loads); 176 rows at 4,160 keys 184, 156, 144. Three planes at head_dim
+// 128 leave shared memory for one group, and passes with a block per chunk
 // (launch_verify) have no use for a second.
 //
 // Softmax: warps w and w + 4 read TMEM lanes 32(w % 4) .. +31, so each thread owns one query
 // vector's row of scores over half the chunk's keys (the two halves exchange their row
 // maxima through shared memory; each keeps its own share of the row sum). The running
-// reference m is raised only when a chunk's maximum exceeds it by more than kLazy (then O in
-// TMEM and l are rescaled); otherwise p = 2^(s - m) <= e^8, and the final o / l does not
+// reference m is raised only when a chunk's maximum exceeds it by more than kLazy (then O
+// and l are rescaled); otherwise p = 2^(s - m) <= e^8, and the final o / l does not
 // depend on the reference. The block's partial (m, l, o) are merged across the cluster
 // through distributed shared memory as in attention.cu, and the normalized output is written
 // as the O projection's hi/lo input.
@@ -41,6 +49,7 @@
 // skips its remaining chunks, waits for its own MMAs in flight and still meets every cluster
 // barrier).
 #include <algorithm>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -65,8 +74,9 @@ constexpr float kLog2e = 1.44269504088896341f;
 
 int g_tc_max_cluster = 8;
 
-// NP: planes of P and V (2: x = hi + lo; 3: hi + mid + lo, fp32's own precision). NG: groups. Each
-// group has its own K, V and P; with two groups P overwrites K, whose products are done by then.
+// NP: planes of Q, K, P and V (2: x = hi + lo; 3: hi + mid + lo, fp32's own precision). NG: groups.
+// Each group has its own K, V and P; with two groups or three planes P overwrites K, whose products
+// are done by then.
 template <int HD, int NP, int NG>
 struct TcSmem {
   static constexpr int KB = HD / 64;                        // 64-wide K blocks of Q and K
@@ -77,10 +87,9 @@ struct TcSmem {
   static constexpr uint32_t V_PLANE = K_PLANE;              // V [64][HD]
   static constexpr uint32_t P_PLANE = TQB * 128;            // P [128][64 keys]
   static constexpr uint32_t Q_OFF = 0;
-  static constexpr uint32_t K_OFF = Q_OFF + 2 * Q_PLANE;
-  static constexpr bool ALIAS = NG > 1;
-  static_assert(!ALIAS || NP * P_PLANE <= 2 * K_PLANE || HD < 128, "P fits over K");
-  static constexpr uint32_t KP = ALIAS && NP * P_PLANE > 2 * K_PLANE ? NP * P_PLANE : 2 * K_PLANE;
+  static constexpr uint32_t K_OFF = Q_OFF + NP * Q_PLANE;
+  static constexpr bool ALIAS = NG > 1 || NP > 2;
+  static constexpr uint32_t KP = NP * (ALIAS && P_PLANE > K_PLANE ? P_PLANE : K_PLANE);   // K, P
   static constexpr uint32_t V_OFF = K_OFF + KP;
   static constexpr uint32_t P_OFF = ALIAS ? K_OFF : V_OFF + NP * V_PLANE;
   static constexpr uint32_t GROUP = KP + NP * V_PLANE + (ALIAS ? 0 : NP * P_PLANE);   // per group
@@ -193,6 +202,38 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
   const int half = tid / TQB;                      //   half of the chunk's keys
   float m_ref = -INFINITY, l_run = 0.f;
   int nproc = 0;                                    // chunks whose P V has been issued
+  // Two planes: O is one chain over the group's chunks in TMEM. Three: every chunk's P V starts
+  // anew, and the threads add it to o_sum, rounded to nearest (this half's columns of row qi).
+  constexpr bool kChain = NP == 2;
+  float o_sum[kChain ? 1 : HD / 32][16];
+#pragma unroll
+  for (int q = 0; q < (kChain ? 0 : HD / 32); ++q)
+#pragma unroll
+    for (int e = 0; e < 16; ++e) o_sum[q][e] = 0.f;
+  // f(n, m, kb, kk, add) for every product of planes n and m with n + m < NP, the smallest first, of
+  // the 16-wide K steps kk of `blocks` 64-wide blocks kb
+  auto each_product = [](auto&& f, auto blocks) {
+#pragma unroll
+    for (int t = NP - 1; t >= 0; --t)
+#pragma unroll
+      for (int kb = 0; kb < blocks(); ++kb)
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+          for (int n = 0; n <= t; ++n) f(n, t - n, kb, kk, t < NP - 1 || (kb | kk | n));
+  };
+  auto add_o = [&] {   // the finished P V (whole warps)
+    if constexpr (!kChain) {
+      tc::tc_fence_after();
+#pragma unroll
+      for (int q = 0; q < HD / 32; ++q) {
+        float o[16];
+        tc::tmem_ld16(t_o + lane_base + half * (HD / 2) + 16 * q, o);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) o_sum[q][e] += o[e];
+      }
+    }
+  };
 
   // Staging is software-pipelined: the group's next K rows (with one group, the V rows too) are
   // loaded from the fp32 cache into registers right after a chunk's score MMAs are issued (in
@@ -258,11 +299,11 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
       const float sc = a.scale * kLog2e;
       const float x[8] = {qr[u][0].x * sc, qr[u][0].y * sc, qr[u][0].z * sc, qr[u][0].w * sc,
                           qr[u][1].x * sc, qr[u][1].y * sc, qr[u][1].z * sc, qr[u][1].w * sc};
-      uint4 p[2];
-      split8<2>(x, p);
+      uint4 p[NP];
+      split8<NP>(x, p);
       const uint32_t off = SM::Q_OFF + (dc >> 3) * SM::Q_KB + tc::sw128_offset(qv, dc & 7);
-      st_shared16(sm, off, p[0]);
-      st_shared16(sm, off + SM::Q_PLANE, p[1]);
+#pragma unroll
+      for (int n = 0; n < NP; ++n) st_shared16(sm, off + n * SM::Q_PLANE, p[n]);
     }
   }
 
@@ -276,8 +317,12 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
     const int t0 = c * ACH;
     if (!kPreV) load_v(i);
     // the group's previous P V has completed: K, V and P may be overwritten
-    if (nproc > 0 && !tc::mbar_wait(&bar_o[grp], (nproc - 1) & 1, a.status, a.wait_ns))
-      failed = true;
+    if (nproc > 0) {
+      bool ok = tc::mbar_wait(&bar_o[grp], (nproc - 1) & 1, a.status, a.wait_ns);
+      if constexpr (!kChain) ok = __all_sync(0xffffffffu, ok);
+      if (!ok) failed = true;
+      else add_o();
+    }
     if (i + NG < nb_chunks) kptrs(i + NG);
     // ---- stage the chunk: split the loaded K and V into hi/lo and store
 #pragma unroll
@@ -285,11 +330,11 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
       const int idx = tid + u * GTHREADS, j = idx / DCH, dc = idx % DCH;
       const float x[8] = {kr[u][0].x, kr[u][0].y, kr[u][0].z, kr[u][0].w,
                           kr[u][1].x, kr[u][1].y, kr[u][1].z, kr[u][1].w};
-      uint4 p[2];
-      split8<2>(x, p);
+      uint4 p[NP];
+      split8<NP>(x, p);
       const uint32_t off = SM::K_OFF + (dc >> 3) * SM::K_KB + tc::sw128_offset(j, dc & 7);
-      st_shared16(smg, off, p[0]);
-      st_shared16(smg, off + SM::K_PLANE, p[1]);
+#pragma unroll
+      for (int n = 0; n < NP; ++n) st_shared16(smg, off + n * SM::K_PLANE, p[n]);
     }
 #pragma unroll
     for (int u = 0; u < K_IT; ++u) {
@@ -304,22 +349,17 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
     }
     tc::fence_proxy_async();
     if (group_failed()) break;
-    // ---- S = Q K^T (hi.hi + hi.lo + lo.hi over the head dimension)
+    // ---- S = Q K^T over the head dimension
     if (tid == kIssuer) {
       tc::tc_fence_after();
-#pragma unroll
-      for (int kb = 0; kb < KB; ++kb) {
-        const uint64_t qh = tc::desc_sw128(sbase + SM::Q_OFF + kb * SM::Q_KB);
-        const uint64_t ql = tc::desc_sw128(sbase + SM::Q_OFF + SM::Q_PLANE + kb * SM::Q_KB);
-        const uint64_t kh = tc::desc_sw128(gbase + SM::K_OFF + kb * SM::K_KB);
-        const uint64_t kl = tc::desc_sw128(gbase + SM::K_OFF + SM::K_PLANE + kb * SM::K_KB);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {   // K = 16 per MMA: +32 bytes = +2 in the descriptor
-          tc::umma_bf16(t_s, qh + 2 * kk, kh + 2 * kk, idesc_s, (kb | kk) ? 1u : 0u);
-          tc::umma_bf16(t_s, qh + 2 * kk, kl + 2 * kk, idesc_s, 1u);
-          tc::umma_bf16(t_s, ql + 2 * kk, kh + 2 * kk, idesc_s, 1u);
-        }
-      }
+      each_product(
+          [&](int n, int m, int kb, int kk, bool add) {   // K = 16: +32 bytes = +2 in the descriptor
+            tc::umma_bf16(
+                t_s, tc::desc_sw128(sbase + SM::Q_OFF + n * SM::Q_PLANE + kb * SM::Q_KB) + 2 * kk,
+                tc::desc_sw128(gbase + SM::K_OFF + m * SM::K_PLANE + kb * SM::K_KB) + 2 * kk, idesc_s,
+                add);
+          },
+          std::integral_constant<int, KB>());
       tc::umma_commit(&bar_s[grp]);
     }
     if (i + NG < nb_chunks) {   // in flight during this chunk's softmax
@@ -370,7 +410,14 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
       }
       // each half rescales its half of the output row's columns, each lane by its own factor
       // (1 where its reference stayed)
-      if (__any_sync(0xffffffffu, rescale_o)) {
+      if constexpr (!kChain) {
+        if (rescale_o) {
+#pragma unroll
+          for (int q = 0; q < HD / 32; ++q)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) o_sum[q][e] *= alpha;
+        }
+      } else if (__any_sync(0xffffffffu, rescale_o)) {
         const float f = rescale_o ? alpha : 1.f;
 #pragma unroll 1
         for (int q = 0; q < HD / 32; ++q) {
@@ -408,24 +455,16 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
       tc::tc_fence_before();
     }
     group_sync();
-    // ---- O += P V over the chunk's 64 keys: hi.hi + hi.lo + lo.hi, or with three planes the six
-    //      products down to 2^-24 of the largest
+    // ---- O = P V over the chunk's 64 keys (kChain: O +=)
     if (tid == kIssuer) {
       tc::tc_fence_after();
-      uint64_t pd[NP], vd[NP];
-#pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        pd[n] = tc::desc_sw128(gbase + SM::P_OFF + n * SM::P_PLANE);
-        vd[n] = tc::desc_sw128_mn(gbase + SM::V_OFF + n * SM::V_PLANE, SM::K_KB);
-      }
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
-#pragma unroll
-        for (int n = 0; n < NP; ++n)
-#pragma unroll
-          for (int m = 0; n + m < NP; ++m)
-            tc::umma_bf16(t_o, pd[n] + 2 * kk, vd[m] + 128 * kk, idesc_o,   // 16 keys: 2 KB
-                          (nproc | kk | n | m) ? 1u : 0u);
+      each_product(
+          [&](int n, int m, int, int kk, bool add) {   // 16 keys: 2 KB of V
+            tc::umma_bf16(t_o, tc::desc_sw128(gbase + SM::P_OFF + n * SM::P_PLANE) + 2 * kk,
+                          tc::desc_sw128_mn(gbase + SM::V_OFF + m * SM::V_PLANE, SM::K_KB) + 128 * kk,
+                          idesc_o, add || (kChain && nproc));
+          },
+          std::integral_constant<int, 1>());
       tc::umma_commit(&bar_o[grp]);
     }
     ++nproc;
@@ -440,8 +479,11 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
   // ---- the block's partial (m, l, o) per query vector into shared memory (o over everything):
   //      each half writes its half of the row's columns; l is the sum of the halves' shares. A
   //      second group leaves its partial there for the first one to add to its own.
-  if (failed || (nproc > 0 && !tc::mbar_wait(&bar_o[grp], (nproc - 1) & 1, a.status, a.wait_ns)))
+  if (failed || (nproc > 0 && !__all_sync(0xffffffffu, tc::mbar_wait(&bar_o[grp], (nproc - 1) & 1,
+                                                                     a.status, a.wait_ns))))
     s_abort[grp] = 1;   // (read after the next barrier, no longer written there)
+  else if (nproc > 0)
+    add_o();
   if (half == 1) s_mx[grp][1][qi] = l_run;
   __syncthreads();
   float* const s_po = reinterpret_cast<float*>(sm);              // [TQB][OP]
@@ -449,13 +491,13 @@ __global__ void __launch_bounds__(NG * GTHREADS, 1) k_attn_tc(AttnArgs a) {
   const bool have_o = nproc > 0 && !s_abort[grp];
   if (have_o) tc::tc_fence_after();
   auto each_o = [&](auto&& put) {   // put(column, 16 values) over this half's columns
-#pragma unroll 1
+#pragma unroll(kChain ? 1 : HD / 32)
     for (int q = 0; q < HD / 32; ++q) {
       const int col = half * (HD / 2) + 16 * q;
       float o[16];
 #pragma unroll
-      for (int e = 0; e < 16; ++e) o[e] = 0.f;
-      if (have_o) tc::tmem_ld16(t_o + lane_base + col, o);   // (uniform over the group)
+      for (int e = 0; e < 16; ++e) o[e] = kChain ? 0.f : o_sum[kChain ? 0 : q][e];
+      if (kChain && have_o) tc::tmem_ld16(t_o + lane_base + col, o);   // (uniform over the group)
       if (qi < nq) put(col, o);
     }
   };
@@ -613,8 +655,7 @@ int configure_attention_tc() {
 }
 
 void launch_attn_tc(const AttnArgs& a, int n_z, cudaStream_t s) {
-  // prefill passes with three planes of P and V: their K/V cache carries every later step (two
-  // planes: 13B logits after two layers 2.1e-5 -> 2.6e-5 off 64 bits, 3 to 7 % of the pass)
+  // prefill passes with three planes
   if (a.n_tchunks == 0)
     a.kv.hd == 128 ? launch_tc<128, 3, 1>(a, n_z, s) : launch_tc<64, 3, 2>(a, n_z, s);
   else
