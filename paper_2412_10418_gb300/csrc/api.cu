@@ -505,7 +505,8 @@ struct AttnPass {
   int rows_per_prompt = 0;            // dense: z = b * qb_count + qb; prefill: of the prompt
                                       //   with the most rows
   const std::vector<int32_t>* zmap = nullptr;  // prefill: (b, qb) pairs for this model, in
-  int qblock = 0;                              //   query blocks of qblock vectors
+  int qblock = 0;                              //   query blocks of qblock vectors that see
+  double avg_chunks = 0;                       //   avg_chunks key chunks on average
   int n_chunks = 0;
   int n_tchunks = 0;                  // tail-key chunks (attn_tail_chunks)
 };
@@ -534,6 +535,7 @@ void forward(cdsl_ctx* c, ModelW& m, const RowPlan& plan, RowDesc* rows, int R, 
     n_z = (int)ap.zmap->size() / 2;
     at.zmap = c->attn_zmap;
     at.qblock = ap.qblock;
+    at.avg_chunks = ap.avg_chunks;
     cudaMemcpyAsync(c->attn_zmap, ap.zmap->data(), ap.zmap->size() * 4, cudaMemcpyHostToDevice, s);
   } else {
     at.qblock = attn_tc ? attn_tc_qblock(ap.rows_per_prompt, at.G, ap.n_tchunks > 0)
@@ -899,11 +901,15 @@ int32_t cdsl_prefill(cdsl_ctx* c, const int32_t* d_prompts, const int32_t* h_pro
       ap->rows_per_prompt = most;
       ap->qblock = use_attn_tc(c, most, G) ? attn_tc_qblock(most, G, false) : attn_qblock();
       // a prompt's last query blocks, which see the most keys, first
-      for (int b = 0; b < B; ++b)
+      double seen = 0;
+      for (int b = 0, first = 0; b < B; first += per_prompt[b++])   // its rows: from `first` on
         for (int q = (per_prompt[b] * G + ap->qblock - 1) / ap->qblock - 1; q >= 0; --q) {
           z.push_back(b);
           z.push_back(q);
+          const int last = std::min(per_prompt[b] * G, (q + 1) * ap->qblock) - 1;   // its last vector
+          seen += (rows[first + last / G].n_prefix + attn_chunk() - 1) / attn_chunk();
         }
+      ap->avg_chunks = seen / (z.size() / 2);
       return z;
     };
     AttnPass apt, apd;

@@ -614,8 +614,9 @@ void launch_tc(const AttnArgs& a, int n_z, cudaStream_t s) {
   const int chunks = a.n_chunks + a.n_tchunks;
   const ClusterFit& f = g_tc_fit<HD, NP, NG>;
   const int groups = a.kv.kvh * n_z;
-  const int cl = a.zmap ? attn_cluster_size_causal(f, g_tc_max_cluster, chunks, groups)
-                        : attn_cluster_size(f, g_tc_max_cluster, chunks, groups);
+  const int cl = a.zmap
+                     ? attn_cluster_size_causal(f, g_tc_max_cluster, chunks, groups, a.avg_chunks)
+                     : attn_cluster_size(f, g_tc_max_cluster, chunks, groups);
   launch_pdl_cluster(k_attn_tc<HD, NP, NG>, dim3(cl, a.kv.kvh, n_z), dim3(NG * GTHREADS),
                      TcSmem<HD, NP, NG>::bytes, cl, s, a);
 }

@@ -78,6 +78,7 @@ struct AttnArgs {
   void* out; size_t plane; float scale;
   int32_t n_chunks, n_tchunks, qb_count, qblock;
   const int32_t* zmap;
+  double avg_chunks;           // with a zmap: chunks that its query blocks see, on average
   int32_t* status;
   unsigned long long* stamp;   // in-graph launch timing record (LaunchStamp), or nullptr
   uint64_t wait_ns;            // limit of the tensor-core kernel's MMA waits (nanoseconds)
