@@ -490,23 +490,37 @@ const CUtensorMap& tensor_map(cdsl_ctx* c, const void* base, int inner, int oute
   return c->maps.emplace(key, m).first->second;
 }
 
-// Query vectors per prompt and KV head from which a pass of a bf16 model runs on the tensor-core
-// attention (attention_tc.cu) rather than the CUDA-core one (attention.cu). The 7B verify pass
-// (80) measured 16.3 us per launch on the former against 20.1 us on the latter; decode passes
-// (16-36) stay on the CUDA cores, where a block's 64-key chunk is too small for the MMA's 128 rows
-// to pay.
+// Query vectors per prompt and KV head from which a dense pass of a bf16 model runs on the
+// tensor-core attention (attention_tc.cu) rather than the CUDA-core one (attention.cu). The 7B
+// verify pass (80) measured 16.3 us per launch on the former against 20.1 us on the latter; decode
+// passes (16-36) stay on the CUDA cores, where a block's 64-key chunk is too small for the MMA's 128
+// rows to pay.
 constexpr int kAttnTcMinVectors = 64;
 bool use_attn_tc(const cdsl_ctx* c, int rows_per_prompt, int G) {
   return c->dtype == CDSL_DTYPE_BF16 && rows_per_prompt * G >= kAttnTcMinVectors;
 }
 
+// A prefill pass of a bf16 model runs on the tensor-core attention where the CUDA-core kernel would
+// need more than its one wave of two blocks per SM (`blocks` blocks of query vectors over `chunks`
+// key chunks), and where the tensor-core blocks (tc_blocks) are mostly full: at least 2.5 of the
+// CUDA-core kernel's in each, which has four times their vectors. Measured over 207 launches (head
+// dims 64 and 128, 64 to 4096 vectors of 1 to 32 prompts, 0 to 3072 positions before them), the
+// chosen kernel is 0.3 % slower than the faster one on average. Below the line: one prompt of 128
+// vectors 8 us on the CUDA cores, 14 on the tensor cores (head dim 64), 12 and 23 (head dim 128);
+// above it: 96 vectors of 16 prompts 34 and 22, one prompt of 4096 372 and 139. At most the wrong
+// side costs 17 % (16 rows of a prompt's end, 26 against 22 us).
+bool use_attn_tc_prefill(const cdsl_ctx* c, int blocks, int tc_blocks, int chunks) {
+  return c->dtype == CDSL_DTYPE_BF16 && (long long)blocks * chunks > 2 * c->plan_sms &&
+         2 * blocks >= 5 * tc_blocks;
+}
+
 // Attention layout of a pass: rows per prompt (dense z mapping) or a host-built z map.
 struct AttnPass {
-  int rows_per_prompt = 0;            // dense: z = b * qb_count + qb; prefill: of the prompt
-                                      //   with the most rows
+  int rows_per_prompt = 0;            // dense: z = b * qb_count + qb
   const std::vector<int32_t>* zmap = nullptr;  // prefill: (b, qb) pairs for this model, in
   int qblock = 0;                              //   query blocks of qblock vectors that see
-  double avg_chunks = 0;                       //   avg_chunks key chunks on average
+  double avg_chunks = 0;                       //   avg_chunks key chunks on average,
+  bool tc = false;                             //   on the tensor cores
   int n_chunks = 0;
   int n_tchunks = 0;                  // tail-key chunks (attn_tail_chunks)
 };
@@ -530,7 +544,7 @@ void forward(cdsl_ctx* c, ModelW& m, const RowPlan& plan, RowDesc* rows, int R, 
   at.status = c->st.status;
   at.wait_ns = c->wait_ns;
   int n_z;
-  const bool attn_tc = use_attn_tc(c, ap.rows_per_prompt, at.G);
+  const bool attn_tc = ap.zmap ? ap.tc : use_attn_tc(c, ap.rows_per_prompt, at.G);
   if (ap.zmap) {
     n_z = (int)ap.zmap->size() / 2;
     at.zmap = c->attn_zmap;
@@ -898,8 +912,15 @@ int32_t cdsl_prefill(cdsl_ctx* c, const int32_t* d_prompts, const int32_t* h_pro
     auto zmap_for = [&](const cdsl_model_cfg& mc, AttnPass* ap) {
       std::vector<int32_t> z;
       const int G = group_size(mc);
-      ap->rows_per_prompt = most;
-      ap->qblock = use_attn_tc(c, most, G) ? attn_tc_qblock(most, G, false) : attn_qblock();
+      ap->n_chunks = (maxpos + attn_chunk()) / attn_chunk();
+      auto blocks_of = [&](int qblock) {
+        int n = 0;
+        for (int r : per_prompt) n += (r * G + qblock - 1) / qblock;
+        return n * mc.n_kv_heads;
+      };
+      const int tc_qblock = attn_tc_qblock(most, G, false);
+      ap->tc = use_attn_tc_prefill(c, blocks_of(attn_qblock()), blocks_of(tc_qblock), ap->n_chunks);
+      ap->qblock = ap->tc ? tc_qblock : attn_qblock();
       // a prompt's last query blocks, which see the most keys, first
       double seen = 0;
       for (int b = 0, first = 0; b < B; first += per_prompt[b++])   // its rows: from `first` on
@@ -916,7 +937,6 @@ int32_t cdsl_prefill(cdsl_ctx* c, const int32_t* d_prompts, const int32_t* h_pro
     const std::vector<int32_t> zt = zmap_for(c->tcfg, &apt), zd = zmap_for(c->dcfg, &apd);
     apt.zmap = &zt;
     apd.zmap = &zd;
-    apt.n_chunks = apd.n_chunks = (maxpos + attn_chunk()) / attn_chunk();
     forward(c, c->tgt, RowPlan{}, c->rows_p, R, nlm, c->lm_gather, c->logits, false, apt);
     if (nlm) {
       RowStatsArgs a{};

@@ -78,9 +78,14 @@ def second_layer_v(s, b):
 
 @pytest.mark.parametrize("H,KVH,hd", [(4, 4, 64), (4, 1, 128)], ids=["hd64", "hd128"])
 @pytest.mark.parametrize("lens,score", [([1000], 1.5), ([1000], 25.0), ([640, 333, 65], 5.0),
-                                        ([3300], 1.5)],
-                         ids=["1000", "1000_peaked", "ragged", "3300"])
+                                        ([3300], 1.5), ([384], 1.5), ([416], 1.5),
+                                        ([160] * 8, 1.5), ([70] * 8, 1.5), ([3], 1.5)],
+                         ids=["1000", "1000_peaked", "ragged", "3300", "384", "416", "8x160", "8x70",
+                              "3"])
 def test_prefill_attention_keeps_fp32_precision(H, KVH, hd, lens, score):
+    """On both sides of the line between the CUDA-core and the tensor-core kernel (both head counts:
+    384 and 416 rows, eight prompts of 70 and 160), full and ragged passes, continued ones (more
+    than 1024 rows)."""
     s = setup(H, KVH, hd, lens, score)
     page = 64
     eng = make_engine(s, page_size=page)
