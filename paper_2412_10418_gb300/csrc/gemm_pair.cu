@@ -16,16 +16,18 @@
 // (16 KB + 256 N bytes) and had room for two stages in flight: here it is four or more.
 //
 // The tensor core truncates when it adds into an fp32 accumulator, so a chain of MMAs shrinks
-// the sum by about 1.8e-8 per K step of 16 and plane (K = 4096 in one chain: 9.2e-6 off, more than
-// the 2.5e-6 of the hi/lo split). A tile's K range is therefore accumulated in segments of at
-// most kSegKb blocks (2.2e-6), into two TMEM accumulator sets in turn; the epilogue warps add each
-// finished segment to fp32 sums in their registers (rounded to nearest) while the next one
-// accumulates (k_gemm_pair<.., true>). A K range of one segment is finished straight from TMEM
-// (<.., false>), and so are gate/up and QKV tiles of more than 128 rows, whose two accumulators
-// leave TMEM no room for a second set: one chain, for gate/up of up to kWideKb blocks (13B, 224
-// rows: 88 us against 115; the kernel before had the same chain there), for QKV of kWideQkvKb. Where TMEM has room (planes == 2)
-// the lo plane accumulates apart, which halves a chain's truncations. 13B logits after two layers,
-// against 64 bits: 2.1e-5 (the kernel before: 2.7e-5; one chain per tile in all shapes: 3.3e-5).
+// the sum: by 1.4e-7 per 64-wide K block, or 6e-8 where the lo plane accumulates apart (planes == 2,
+// where TMEM has room), over K = 4096 in one chain 8.8e-6 where the hi/lo split of the activations
+// leaves 2.4e-6. A tile's K range is therefore accumulated in chains of at most chain_blocks() blocks,
+// into two TMEM accumulator sets in turn; the epilogue warps add each finished chain to fp32 sums in
+// their registers (rounded to nearest) while the next one accumulates (k_gemm_pair<.., true>). A K
+// range of one chain is finished straight from TMEM (<.., false>). The bound is the rounding error
+// of a serial fp32 sum of K products, 1.8e-8 sqrt(K) as measured on the CUDA-core GEMM: 1.1e-6 at
+// K = 4096, in chains of 8 blocks or 16 with lo apart. Logits against 64 bits (mean of six seeds;
+// the kernels before, which took one chain per tile up to 256 rows and the CUDA cores above): 13B
+// slice at 224 rows 1.5e-5 (2.7e-5), 7B slice at 320 rows 1.3e-5 (1.4e-5), small model at 640 rows
+// 6.3e-6 (6.4e-6). Gate/up tiles of 129 to 256 rows in one chain of all 80 blocks, which leave TMEM
+// no room for a second set, were faster (13B, 224 rows: 90 us against 126) but 2.3e-5 off each.
 //
 // Schedule (plan_pair): the tiles of a launch are dealt to the pairs in turn (persistent), or,
 // with few tiles, a cluster of S pairs splits a tile's K range: the partial tiles go to shared
@@ -44,6 +46,7 @@
 // ran out lands the copies of both its CTAs before either leaves: the leader completes the
 // transaction counts of stages that only one of them filled.
 #include <algorithm>
+#include <cmath>
 
 #include "gemm.cuh"
 #include "kernels.h"
@@ -53,18 +56,20 @@ namespace cdsl {
 namespace {
 
 constexpr int kStagesMax = 8;
-constexpr int kEpWarps = 16;          // (1024 rows, 7B gate/up: 231 us with 8, 223 with 12, 219 with 16;
-                                     //  256 rows, 13B O: 30.1, 28.1, 27.4)
+constexpr int kEpWarps = 16;          // (256 rows, 13B O: 30.1 us with 8, 28.1 with 12, 27.4 with 16)
 constexpr int kEpThreads = kEpWarps * 32;
 constexpr int kThreads = 64 + kEpThreads;
 constexpr int kGroups = kEpWarps / 4;   // warps that share 32 TMEM lanes
 constexpr int kChunks = 16 / kGroups;   // groups of 16 columns a warp sums
-constexpr int kSegKb = 16;           // 64-wide K blocks per accumulation chain (at most)
-constexpr int kWideKb = 80;          //   and of a tile's one chain that fills TMEM: gate/up,
-constexpr int kWideQkvKb = 24;       //   QKV
 constexpr int kNMax = 256;
 constexpr int kSplitMax = 4;         // pairs per cluster (8 CTAs: the portable cluster size)
 constexpr size_t kSmemMax = 216 * 1024;   // dynamic shared memory a plan may use
+
+// 64-wide K blocks per accumulation chain, at most (its truncation against the rounding of a serial
+// fp32 sum of K products: see above; 4 where that would ask for fewer).
+int chain_blocks(int K, int planes) {
+  return planes * std::max(4, (int)(0.131 * std::sqrt((double)K)));
+}
 
 // Accumulators per tile: gate and up, or the two halves of RoPE pairs.
 constexpr int accs(int mode) { return mode == EPI_SWIGLU || mode == EPI_QKV ? 2 : 1; }
@@ -137,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int tiles = p.m_tiles * NT;
   const int kb0 = q * KBT / S, kb1 = (q + 1) * KBT / S, nkb = kb1 - kb0;
   const int my_tiles = cid < tiles ? (tiles - cid + CN - 1) / CN : 0;
-  const int nseg = kSeg ? (nkb + kSegKb - 1) / kSegKb : 1;   // accumulation chains per tile
+  const int nseg = kSeg ? (nkb + p.chain - 1) / p.chain : 1;   // accumulation chains per tile
   const int n_units = my_tiles * nkb;
   const int pre = min(ST, n_units);
   const uint32_t cols = pow2_cols(p.bufs * p.planes * MT * N);
@@ -380,39 +385,32 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (S > 1) {
     // ---- split K (one tile per cluster): the partial tiles go to shared memory, [accumulator][row]
     //      [128 features], and CTA q of each half finishes rows [q n / S, (q + 1) n / S) of its 128
-    //      weight rows -- in two rounds of half the columns each where a partial tile does not
-    //      fit (p.rounds)
+    //      weight rows
     const bool gave_up =
         warp >= 2 ? tc::named_barrier_or(1, kEpThreads, s_abort != 0) : true;
     const int quarter = warp & 3, cg = (warp - 2) >> 2;
     const int tm = cid / NT, tn = cid % NT;
-    const int r0 = tn * N, rows = min(N, a.R - r0), NH = N / p.rounds;
+    const int r0 = tn * N, rows = min(N, a.R - r0);
     const int L = half * 128 + quarter * 32 + lane;
     const uint32_t mine = tc::smem_u32(smem) + (quarter * 32 + lane) * 4;
-    for (int rd = 0; rd < p.rounds; ++rd) {
-      const int b0 = rd * NH, n = max(0, min(rows - b0, NH));   // this round's columns
-      if (rd > 0) {   // the previous round's partials have been read
-        tc::cluster_arrive();
-        tc::cluster_wait();
-      }
-      if (!kSeg && !gave_up) {
-        float* const part = reinterpret_cast<float*>(smem) + quarter * 32 + lane;
-        const uint32_t d = tmem + ((uint32_t)(quarter * 32) << 16);
-        tc::tc_fence_after();
-        for (int c = cg * 16; c < n; c += 16 * kGroups) {
+    if (!kSeg && !gave_up) {
+      float* const part = reinterpret_cast<float*>(smem) + quarter * 32 + lane;
+      const uint32_t d = tmem + ((uint32_t)(quarter * 32) << 16);
+      tc::tc_fence_after();
+      for (int c = cg * 16; c < rows; c += 16 * kGroups) {
 #pragma unroll
-          for (int m = 0; m < MT; ++m) {
-            float y[16];
-            load_sums(d + m * N + b0 + c, lo, y);
+        for (int m = 0; m < MT; ++m) {
+          float y[16];
+          load_sums(d + m * N + c, lo, y);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) part[(size_t)(m * NH + c + i) * 128] = y[i];
-          }
+          for (int i = 0; i < 16; ++i) part[(size_t)(m * N + c + i) * 128] = y[i];
         }
       }
-      tc::cluster_arrive();   // this CTA's partial is complete (release)
-      tc::cluster_wait();     // every CTA's is (acquire)
-      if (gave_up) continue;
-      const int ra = q * n / S, rb = (q + 1) * n / S;
+    }
+    tc::cluster_arrive();   // this CTA's partial is complete (release)
+    tc::cluster_wait();     // every CTA's is (acquire)
+    if (!gave_up) {
+      const int ra = q * rows / S, rb = (q + 1) * rows / S;
       for (int c = ra + cg * 8; c < rb; c += 8 * kGroups) {
         float y0[8], y1[8];
 #pragma unroll
@@ -423,11 +421,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int i = 0; i < 8; ++i) {
             const int ci = min(i, rb - 1 - c) * 512;   // (past the share: any row, unused)
             y0[i] += tc::ld_cluster_f32(src + ci);
-            if constexpr (MT == 2) y1[i] += tc::ld_cluster_f32(src + NH * 512 + ci);
+            if constexpr (MT == 2) y1[i] += tc::ld_cluster_f32(src + N * 512 + ci);
           }
         }
-        finish_rows<MODE, 8>(a, tm * 256 + L, r0 + b0 + c, min(8, rb - c), y0, y1, s_rs + b0 + c,
-                             s_qkv + (MODE == EPI_QKV ? b0 + c : 0));
+        finish_rows<MODE, 8>(a, tm * 256 + L, r0 + c, min(8, rb - c), y0, y1, s_rs + c,
+                             s_qkv + (MODE == EPI_QKV ? c : 0));
       }
     }
   }
@@ -498,20 +496,20 @@ PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt
       if (slots < 1 || (S > 1 && tiles > slots)) continue;
       const int clusters = std::min(tiles, slots);
       const int waves = (tiles + clusters - 1) / clusters;
-      // accumulation chains: a second accumulator set to fill while one drains, or one long
-      // chain where the tile's accumulators leave TMEM no room for it
+      // One accumulation chain where that is short enough, its lo plane apart where TMEM has room
+      // (rather than a second set), and a second set to fill while one drains where there are
+      // several tiles and room for both. Else several chains, which need two sets.
       const int nkb = (KBT + S - 1) / S;
-      const bool wide = MT * N > 256, seg = nkb > kSegKb && !wide;
-      if (wide && (nkb <= kSegKb ? S == 1 : nkb > (mode == EPI_SWIGLU ? kWideKb : kWideQkvKb)))
-        continue;
-      // short chains keep lo apart rather than a second set where TMEM has no room for both
-      const int bufs = wide || (!seg && (waves == 1 || 4 * MT * N > 512)) ? 1 : 2;
+      int planes = 2 * MT * N <= 512 ? 2 : 1, bufs = waves > 1 && 4 * MT * N <= 512 ? 2 : 1;
+      const bool seg = nkb > chain_blocks(K, planes);
+      if (seg) {
+        if (2 * MT * N > 512) continue;
+        bufs = 2;
+        planes = 4 * MT * N <= 512 ? 2 : 1;
+      }
+      const int chain = chain_blocks(K, planes);
       const int stages = (int)std::min<size_t>(kStagesMax, (kSmemMax - 1024) / stage);
-      // a split's partial tiles reuse the stages, in two rounds if need be
-      const size_t part = (size_t)MT * N * 512, room = (size_t)stages * stage;
-      const int rounds = S == 1 || part <= room ? 1 : 2;
-      if (S > 1 && (part > rounds * room || (rounds == 2 && seg))) continue;
-      const int planes = 2 * bufs * MT * N <= 512 ? 2 : 1;
+      if (S > 1 && (size_t)MT * N * 512 > stages * stage) continue;   // its partial tiles reuse them
       // Estimated clocks, fitted to 1,500 measured plans (19 projection shapes of the 7B, 13B,
       // 1B and small models, 72 to 1024 rows; the chosen plan is on average 0.9 % slower than
       // the fastest of its shape): a K block costs the MMAs or the fetch of its operands (36
@@ -526,11 +524,11 @@ PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt
       cost = std::max(cost, 2.0 * n_virtual * K / (22.0 * ctas)) + 33.0 * ctas;
       if (seg) cost += 5500;
       if (S == 1) cost += bufs == 1 ? waves * ep : ep;
-      else cost += 260.0 * S + 21.0 * MT * N + 0.2 * ep / S + 10500.0 * (rounds - 1);
+      else cost += 260.0 * S + 21.0 * MT * N + 0.2 * ep / S;
       if (best_cost < 0 || cost < best_cost) {
         best_cost = cost;
-        best = PairPlan{N, nt, m_tiles, KBT, S, stages, bufs, seg, planes, rounds, clusters * 2 * S,
-                        (size_t)stages * stage + 1024};
+        best = PairPlan{N, nt, m_tiles, KBT, S, stages, bufs, seg, chain, planes,
+                        clusters * 2 * S, (size_t)stages * stage + 1024};
       }
     }
   }

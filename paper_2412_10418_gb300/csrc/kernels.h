@@ -182,11 +182,13 @@ void launch_gemm_tc(const TcMaps& maps, const GemmArgs& a, const TcPlan& p, floa
 // tiles of 256 weight rows (times two accumulators for QKV and gate/up) x n activation rows.
 // maps: weight boxes of 64 features x pair_box_rows() rows, activation boxes of 64 x n / 2.
 // n_tiles tiles of n rows cover the pass; split: pairs per cluster sharing a tile's K range;
-// bufs: accumulator sets in TMEM; seg: a tile's K range in several accumulation chains; planes:
-// 2 where hi and lo accumulate apart; rounds: in which a split exchanges its partial tiles. No
-// scratch.
+// bufs: accumulator sets in TMEM; seg: a tile's K range in several accumulation chains, of at most
+// `chain` K blocks; planes: 2 where hi and lo accumulate apart. No scratch.
 constexpr int kPairRows = 64;
-struct PairPlan { int n, n_tiles, m_tiles, kb_total, split, stages, bufs, seg, planes, rounds, ctas; size_t smem; };
+struct PairPlan {
+  int n, n_tiles, m_tiles, kb_total, split, stages, bufs, seg, chain, planes, ctas;
+  size_t smem;
+};
 PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt = 0,
                    int force_split = 0);
 int pair_box_rows(int mode, int hd);

@@ -78,3 +78,77 @@ def test_prefill_passes_of_many_row_tiles(lens):
                       draft=synth.ModelShape(vocab=HD64.vocab, **DRAFT), batch=8, k=2, d=2,
                       prompt_len=260, max_new=8)
     run_parity(make_setup(wl, lens=lens), steps=1, tol=TOL, tol_r=TOL, max_chunk=4096)
+
+
+def exactness_engine(D, d_ffn, batch, k, d, ffn_scale):
+    """One layer of zero attention output; the FFN's output ffn_scale times the embedding's norm (0:
+    none). Returns the engine after verify, its logits and the same in float64."""
+    import torch
+    import paper_2412_10418_gb300 as cdsl
+
+    V = 32000
+    shape = synth.ModelShape(n_layers=1, d_model=D, n_heads=D // 128, n_kv_heads=2 if D == 768 else 4,
+                             d_ffn=d_ffn, vocab=V)
+    small = synth.ModelShape(n_layers=1, d_model=128, n_heads=2, n_kv_heads=1, d_ffn=192, vocab=V)
+    g = torch.Generator(device="cuda").manual_seed(D + d_ffn + batch * k * d)
+
+    def weights(sh):
+        out = {}
+        for name, s in sh.weight_specs():
+            w = torch.ones(s, device="cuda") if len(s) == 1 else torch.randn(
+                s, generator=g, device="cuda")
+            out[name] = (w if len(s) == 1 else w * s[1] ** -0.5).bfloat16()
+        return out
+
+    tw, dw = weights(shape), weights(small)
+    for name in ("l0.ffn_norm", "final_norm"):
+        tw[name] = (1 + 0.1 * torch.randn(D, generator=g, device="cuda")).bfloat16()
+    tw["l0.wo"].zero_()
+    tw["embed"].mul_(D ** 0.5)          # of unit rms; the FFN's output: about 0.35 before the scale
+    tw["l0.w_down"].mul_(ffn_scale / 0.35)
+    eng = cdsl.Engine(shape, small, synth.DTYPE_BF16, [tw[n] for n, _ in shape.weight_specs()],
+                      [dw[n] for n, _ in small.weight_specs()], batch=batch, k=k, d=d, max_prompt=8,
+                      max_new=4, n_keywords=1, a_t=0.3, r_t=0.3)
+    prompts = torch.randint(0, V, (batch, 8), generator=g, device="cuda")
+    torch.cuda.synchronize()   # (the engine works on a stream of its own)
+    eng.prefill(prompts, [8] * batch, torch.zeros(batch, 1, dtype=torch.int32))
+    eng.lookahead()
+    got = torch.empty(batch, k, d + 1, V, device="cuda")
+    eng.verify(got)
+    eng.stream.synchronize()
+    assert eng.status() == 0
+    tok = torch.cat([eng.roots[..., None], eng.draft_tok], -1).long()
+    norm = lambda x: x * torch.rsqrt(x.pow(2).mean(-1, keepdim=True) + shape.norm_eps)
+    h = tw["embed"][tok].double()
+    x = norm(h) * tw["l0.ffn_norm"].double()
+    a = torch.nn.functional.silu(x @ tw["l0.w_gate"].double().T) * (x @ tw["l0.w_up"].double().T)
+    h = h + a @ tw["l0.w_down"].double().T
+    return got, norm(h) * tw["final_norm"].double() @ tw["lm_head"].double().T
+
+
+@pytest.mark.parametrize("D", [768, 4096])
+@pytest.mark.parametrize("batch,k,d", [(1, 13, 4), (1, 16, 9), (1, 16, 13), (2, 16, 9), (4, 16, 15)],
+                         ids=["65rows", "160rows", "224rows", "320rows", "1024rows"])
+def test_sums_are_as_exact_as_a_serial_fp32_sum(D, batch, k, d):
+    """Logits of a model that is its embedding and its LM head: a bf16 embedding times a bf16 gain has
+    16 bits, which the hi and lo planes hold exactly, so what is off is the sum over K alone (and the
+    row's scale, 1e-7). The bound is the rounding of a serial fp32 sum, 1.8e-8 sqrt(K), or the 5.6e-7
+    that chains of four K blocks may take."""
+    got, want = exactness_engine(D, 64, batch, k, d, 0.0)
+    rel = float((got.double() - want).norm() / want.norm())
+    bound = max(1.8e-8 * D ** 0.5, 5.6e-7) + 1e-7
+    print(f"K {D}, {batch * k * (d + 1)} rows: {rel:.2e}, bound {bound:.2e}")
+    assert rel <= bound
+
+
+@pytest.mark.parametrize("batch,k,d", [(1, 13, 4), (1, 16, 9), (1, 16, 13), (4, 16, 15)],
+                         ids=["65rows", "160rows", "224rows", "1024rows"])
+def test_gate_up_sums_do_not_shrink(batch, k, d):
+    """An FFN whose output is as large as the embedding that it is added to: where gate and up fall
+    short by s each, the hidden state turns by about s. Two roundings to hi and lo planes (the
+    activation, 2.4e-6 of half of the state's square, and the LM head's input, 2.4e-6) leave 3e-6;
+    5e-6 is the bound. Gate and up in one chain over K = 4096 are 7e-6 off and more."""
+    got, want = exactness_engine(4096, 11008, batch, k, d, 1.0)
+    rel = float((got.double() - want).norm() / want.norm())
+    print(f"{batch * k * (d + 1)} rows: {rel:.2e}")
+    assert rel <= 5e-6
