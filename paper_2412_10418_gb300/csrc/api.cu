@@ -431,7 +431,7 @@ void gemm(cdsl_ctx* c, const GemmArgs& a) {
     const bool pair = a.R > kPairRows;
     const TcPlan p = pair ? TcPlan{} : plan_tc(a.K, a.n_virtual, a.R, c->plan_sms);
     const PairPlan pp =
-        pair ? plan_pair(a.mode, a.K, a.n_virtual, a.R, c->plan_sms) : PairPlan{};
+        pair ? plan_pair(a.mode, a.K, a.n_virtual, a.R) : PairPlan{};
     // (carve() sizes both over every plan: a launch that would pass them is refused)
     if (!pair && (tc_scratch_floats(p) > c->part_floats || (size_t)p.tiles > c->part_tiles)) {
       c->scratch_short = true;

@@ -13,7 +13,8 @@
 // What bounds it: above about 100 rows the tensor pipe (hi and lo double the MMA work). A
 // 64-wide K block takes 4 N clocks per accumulator; a CTA fetches 16 KB of weights and 128 N
 // bytes of activations for it, 48 bytes per clock at N = 256, where one CTA per tile needs 80
-// (16 KB + 256 N bytes) and had room for two stages in flight: here it is four or more.
+// (16 KB + 256 N bytes) and had room for two stages in flight: here it is four or more (three where
+// a tile with two accumulators takes 256 rows).
 //
 // The tensor core truncates when it adds into an fp32 accumulator, so a chain of MMAs shrinks
 // the sum: by 1.4e-7 per 64-wide K block, or 6e-8 where the lo plane accumulates apart (planes == 2,
@@ -457,8 +458,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 1) tc::tmem_dealloc_pair(tmem, cols);
 }
 
-ClusterFit g_fit;         // cluster residency with a plan's largest shared memory
-bool g_ready = false;
+ClusterFit g_fit;   // cluster residency with a plan's largest shared memory (configure_gemm_pair)
 
 template <typename F>
 void for_modes(F&& f) {
@@ -474,8 +474,7 @@ void for_modes(F&& f) {
 
 }  // namespace
 
-PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt,
-                   int force_split) {
+PairPlan plan_pair(int mode, int K, int n_virtual, int R) {
   const int MT = accs(mode);
   const int m_tiles = (n_virtual + 256 * MT - 1) / (256 * MT), KBT = K / 64;
   PairPlan best{};
@@ -484,15 +483,13 @@ PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt
   // (tiles of 128 rows are always among them: two accumulators of more rows may not be allowed)
   const int nt_max = std::max(nt_min + 7, (R + 127) / 128);
   for (int nt = nt_min; nt <= nt_max; ++nt) {
-    if (force_nt && nt != force_nt) continue;
     const int N = ((R + nt - 1) / nt + 31) / 32 * 32;
     if (N > kNMax || (nt > nt_min && N < 32) || (nt - 1) * N >= R) continue;
     const size_t stage = MT * 16384 + 128 * (size_t)N;
     const int tiles = m_tiles * nt;
     for (int S = 1; S <= kSplitMax; ++S) {
-      if (force_split && S != force_split) continue;
       if (S > 1 && S > KBT) continue;
-      const int slots = g_ready ? g_fit.active[2 * S] : n_sm / (2 * S);
+      const int slots = g_fit.active[2 * S];
       if (slots < 1 || (S > 1 && tiles > slots)) continue;
       const int clusters = std::min(tiles, slots);
       const int waves = (tiles + clusters - 1) / clusters;
@@ -545,8 +542,7 @@ int configure_gemm_pair() {
   cudaGetLastError();
   if (rc) return rc;
   fill_cluster_fit(&g_fit, k_gemm_pair<EPI_STORE, false>, kThreads, kSmemMax, 2 * kSplitMax);
-  g_ready = g_fit.active[2] > 0;
-  return g_ready ? 0 : -1;
+  return g_fit.active[2] > 0 ? 0 : -1;
 }
 
 int pair_box_rows(int mode, int hd) { return mode == EPI_QKV ? hd / 2 : 128; }

@@ -189,8 +189,7 @@ struct PairPlan {
   int n, n_tiles, m_tiles, kb_total, split, stages, bufs, seg, chain, planes, ctas;
   size_t smem;
 };
-PairPlan plan_pair(int mode, int K, int n_virtual, int R, int n_sm, int force_nt = 0,
-                   int force_split = 0);
+PairPlan plan_pair(int mode, int K, int n_virtual, int R);
 int pair_box_rows(int mode, int hd);
 int configure_gemm_pair();
 void launch_gemm_pair(const TcMaps& maps, const GemmArgs& a, const PairPlan& p, cudaStream_t s);

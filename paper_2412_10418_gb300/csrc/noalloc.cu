@@ -54,28 +54,6 @@ __device__ __forceinline__ uint64_t bf16x2_to_f32x2(uint32_t u) {
   return (uint64_t)(u << 16) | ((uint64_t)(u & 0xffff0000u) << 32);
 }
 
-// Sum v[i] over the lanes; lane l then holds the sum of index l / 2 in v[0].
-__device__ __forceinline__ void reduce16(float (&v)[kSums]) {
-  int n = kSums;
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    if (n > 1) {
-      const bool upper = (threadIdx.x & off) != 0;
-#pragma unroll
-      for (int i = 0; i < kSums / 2; ++i) {
-        if (i < n / 2) {
-          const float send = upper ? v[i] : v[i + n / 2];
-          const float keep = upper ? v[i + n / 2] : v[i];
-          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-      }
-      n >>= 1;
-    } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
-    }
-  }
-}
-
 // y[r, n] = sum_k x[r, k] w[n, k], R <= RM rows of x. kw (1, 2, 4 or 8) warps side by side along
 // K, the other 8 / kw over the block's groups of 16 / RM rows of W. Dynamic shared memory:
 // [groups][kw][16] floats.
@@ -135,7 +113,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
       for (int i = 0; i < kSums; ++i)
         s[i] = __uint_as_float((uint32_t)acc[i]) + __uint_as_float((uint32_t)(acc[i] >> 32));
-      reduce16(s);
+      warp_sums<kSums>(s);            // lane l: the sum of index l / 2 in s[0]
       if ((lane & 1) == 0) {          // this warp's own slot: K steps add up in order
         float* dst = red + ((size_t)g * kw + kwi) * kSums + (lane >> 1);
         *dst = kb == 0 ? s[0] : *dst + s[0];
