@@ -162,7 +162,7 @@ def test_get_step1_needs_a_context(cdsl):
 
 @pytest.mark.parametrize("R,K,N,offset", [
     (0, 768, 32000, 0),       # no rows
-    (9, 768, 32000, 0),       # more rows than the fixed scratch holds
+    (9, 768, 32000, 0),       # more than 8 rows
     (4, 8200, 1000, 0),       # K beyond 8192
     (4, 4, 1000, 0),          # K below 8
     (4, 772, 1000, 0),        # K not a multiple of 8
@@ -171,7 +171,7 @@ def test_get_step1_needs_a_context(cdsl):
     (4, 768, 1000, 8),        # misaligned pointers
 ])
 def test_gemv_noalloc_rejects_before_any_cuda_call(cdsl, R, K, N, offset):
-    """Sizes beyond the fixed scratch and misaligned pointers return CDSL_EINVAL from the
+    """Sizes beyond the limits and misaligned pointers return CDSL_EINVAL from the
     host-side checks, before the library touches CUDA (the pointers are never dereferenced)."""
     lib = cdsl.lib()
     base = 1 << 20

@@ -84,17 +84,25 @@ def test_expired_waits_latch_etimeout_and_the_device_stays_usable():
     eng2.close()
 
 
-def test_expired_waits_in_the_large_row_gemm_and_tensor_core_attention():
-    """The same with k = 8, d = 8: 72 verify rows, so the projections run the large-row GEMM
-    (more than 64 rows: stream-K with the contributors' shared fixup, whose counter waits are
-    bounded too) and the verify attention runs on the tensor cores (72 query vectors per KV
-    head). Every block gives up or finishes, the launches end, and a new context on the same
-    device matches the oracle at this shape."""
+WIDE = synth.ModelShape(n_layers=2, d_model=1920, n_heads=30, n_kv_heads=3, d_ffn=3136, vocab=1032)
+DRAFT = synth.ModelShape(n_layers=1, d_model=128, n_heads=2, n_kv_heads=1, d_ffn=192, vocab=1032)
+
+
+@pytest.mark.parametrize("wl", [synth.scaled(synth.SMALL, batch=1, k=8, d=8, max_new=8),
+                                synth.scaled(synth.TINY, dtype=synth.DTYPE_BF16, target=WIDE, draft=DRAFT,
+                                             batch=4, k=13, d=4, prompt_len=9, max_new=8)],
+                         ids=["72rows", "260rows"])
+def test_expired_waits_in_the_large_row_gemm_and_tensor_core_attention(wl):
+    """The same with more than 64 verify rows, where the projections run on pairs of SMs (72 rows of
+    the small model: clusters of three and four pairs that split K; 260 rows of d_model 1920: also
+    whole K ranges in several accumulation chains) and the verify attention on the tensor cores. The
+    pairs land the copies of both their blocks before either leaves, the clusters meet every barrier,
+    the launches end, and a new context on the same device matches the oracle at this shape."""
     import torch
     import paper_2412_10418_gb300 as cdsl
     from cdsl_parity import run_parity
 
-    s = make_setup(synth.scaled(synth.SMALL, batch=1, k=8, d=8, max_new=8))
+    s = make_setup(wl)
     eng = engine(s)
     eng.step()
     assert eng.status() == cdsl.CDSL_OK

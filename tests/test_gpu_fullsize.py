@@ -61,7 +61,7 @@ def test_7b_full_depth_bench_configuration():
 
 def test_13b_shapes_bench_configuration():
     """13B-shaped target (GQA 40/8, FFN 13824) with the 1B-shaped draft, 4 prompts of 1024
-    tokens, k = 8, d = 6: 224 verify rows (two MMAs per K step: hi and lo no longer fit one)."""
+    tokens, k = 8, d = 6: 224 verify rows (the paired GEMM, attention of three query blocks)."""
     check(synth.THIRTEEN_B_SLICE, steps=2)
 
 

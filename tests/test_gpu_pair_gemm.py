@@ -36,6 +36,28 @@ def test_verify_rows_at_tile_edges(shape, batch, k, d):
     run_parity(make_setup(wl), steps=2, tol=TOL, tol_r=TOL)
 
 
+def ragged(hd, heads, kv_heads, d_ffn):
+    return synth.ModelShape(n_layers=2, d_model=hd * heads, n_heads=heads, n_kv_heads=kv_heads,
+                            d_ffn=d_ffn, vocab=1032)
+
+
+@pytest.mark.parametrize("shape,batch", [(ragged(64, 30, 3, 3136), 1), (ragged(64, 30, 3, 3136), 2),
+                                         (ragged(64, 30, 3, 3136), 4), (ragged(64, 30, 3, 3136), 8),
+                                         (ragged(128, 15, 5, 3136), 1), (ragged(128, 15, 5, 3136), 4),
+                                         (ragged(64, 17, 17, 8512), 1), (ragged(64, 17, 17, 8512), 4)],
+                         ids=lambda v: f"{v.d_model}x{v.d_ffn}" if hasattr(v, "d_ffn") else f"{65 * v}rows")
+def test_chains_and_splits_on_ragged_shapes(shape, batch):
+    """K ranges of 17 to 133 blocks, whole and split over two to four pairs, in one chain and in
+    several of uneven lengths, their lo planes apart and not; features and rows that fill neither
+    the weight tiles nor the row tiles. (On 152 SMs: gate/up whole in chains of 4, 5 and 10 blocks, in
+    two in chains of 4 and 5 and in four; down in two to four with chains of 7, 12 and 24 and without;
+    QKV and O in two with chains, in three and four without.)"""
+    wl = synth.scaled(synth.TINY, dtype=synth.DTYPE_BF16, target=shape,
+                      draft=synth.ModelShape(vocab=shape.vocab, **DRAFT), batch=batch, k=13, d=4,
+                      prompt_len=9, max_new=8, reward_head=True)
+    run_parity(make_setup(wl), steps=1, tol=TOL, tol_r=TOL)
+
+
 @pytest.mark.parametrize("shape", [HD64, HD128], ids=["hd64", "hd128"])
 @pytest.mark.parametrize("batch,k,d", [(1, 15, 1), (1, 12, 2), (1, 16, 3)],
                          ids=["30rows", "36rows", "64rows"])

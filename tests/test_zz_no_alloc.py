@@ -3,11 +3,11 @@ product computed by torch, and against the step library's own verify pass.
 
 Some callers of this library cannot allocate device memory: host frameworks whose caching
 allocator already holds the GPU's memory, real-time loops that must not block on cudaMalloc,
-runtimes that forbid device allocation after start-up. cdsl_gemv_noalloc serves them: its
-scratch is a fixed array inside the library. The first test checks it against x @ w^T in fp64
-over every row count it takes (1..8), outputs that are not a multiple of the 128-row tile,
+runtimes that forbid device allocation after start-up. cdsl_gemv_noalloc serves them: one kernel
+without scratch in global memory. The first test checks it against x @ w^T in fp64
+over every row count it takes (1..8), outputs that do not divide among the blocks,
 inputs that are not a multiple of the 256-wide K step and the 8192 K limit, at 2e-5 of the
-sum of |x||w| (the hi/lo split of x keeps about 17 bits; the products and sums are fp32).
+sum of |x||w| (products and sums are fp32; tests/test_gpu_simt_gemm.py has the tight bound).
 The second builds a bf16 model whose layers leave the residual stream unchanged (the
 attention-output and FFN-down projections are zero), so cdsl_verify's logits are
 lm_head(RMSNorm(E[token])) for every verify row; it recomputes those normalized rows in fp32
@@ -23,7 +23,7 @@ from cdsl_parity import make_engine, make_setup
 pytestmark = pytest.mark.gpu
 
 TOL16 = 2e-2   # the bf16 logits tolerance of the parity tests
-REL = 2e-5     # of sum_k |x_k| |w_k|: the hi/lo split and fp32 accumulation
+REL = 2e-5     # of sum_k |x_k| |w_k|
 
 
 @pytest.mark.parametrize("R,K,N", [(1, 768, 1000), (2, 1000, 129), (3, 2048, 3072),
@@ -42,7 +42,7 @@ def test_noalloc_gemv_matches_fp64_product(R, K, N):
     bound = REL * (x.double().abs() @ w.double().abs().t()) + 1e-30
     stream = torch.cuda.current_stream()
     outs = []
-    for _ in range(2):                      # two calls in a row share the scratch
+    for _ in range(2):                      # two calls in a row give the same bits
         y = torch.full((R, N), float("nan"), dtype=torch.float32, device="cuda")
         cdsl.cdsl_gemv_noalloc(w, x, y, stream.cuda_stream)
         stream.synchronize()
@@ -95,9 +95,9 @@ def test_noalloc_gemv_matches_verify_logits():
         err = float((y - want).abs().max())
         assert err <= TOL16, f"max |diff| {err}"
         results.append(y)
-    assert torch.equal(results[0], results[1])   # fixed-order split-K sum: same bits again
+    assert torch.equal(results[0], results[1])   # fixed-order sums: same bits again
 
-    # sizes beyond the fixed scratch are refused before anything is launched
+    # sizes beyond its limits are refused before anything is launched
     big = torch.zeros((9, 768), dtype=torch.float32, device="cuda")
     with pytest.raises(cdsl.CdslError) as e:
         cdsl.cdsl_gemv_noalloc(w, big, torch.empty((9, V), device="cuda"), stream.cuda_stream)
