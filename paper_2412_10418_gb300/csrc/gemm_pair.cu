@@ -24,7 +24,7 @@
 // their registers (rounded to nearest) while the next one accumulates (k_gemm_pair<.., true>). A K
 // range of one chain is finished straight from TMEM (<.., false>). The bound is the rounding error
 // of a serial fp32 sum of K products, 1.8e-8 sqrt(K) as measured on the CUDA-core GEMM: 1.1e-6 at
-// K = 4096, in chains of 8 blocks or 16 with lo apart. Logits against 64 bits (mean of six seeds;
+// K = 4096, in chains of 8 blocks, or 12 with lo apart (7e-7). Logits against 64 bits (mean of six seeds;
 // the kernels before, which took one chain per tile up to 256 rows and the CUDA cores above): 13B
 // slice at 224 rows 1.5e-5 (2.7e-5), 7B slice at 320 rows 1.3e-5 (1.4e-5), small model at 640 rows
 // 6.3e-6 (6.4e-6). Gate/up tiles of 129 to 256 rows in one chain of all 80 blocks, which leave TMEM
@@ -67,9 +67,13 @@ constexpr int kSplitMax = 4;         // pairs per cluster (8 CTAs: the portable 
 constexpr size_t kSmemMax = 216 * 1024;   // dynamic shared memory a plan may use
 
 // 64-wide K blocks per accumulation chain, at most (its truncation against the rounding of a serial
-// fp32 sum of K products: see above; 4 where that would ask for fewer).
+// fp32 sum of K products: see above; 4 where that would ask for fewer). Half as many again with lo
+// apart: twice as many keep the bound too, but the small model's short prompts, whose projections of
+// up to 128 rows had run in splits of 4 blocks, were 1 % further off than before (logits 6.13e-6
+// against 6.07e-6, now 6.05e-6; its first step of 32 prompts 7.64 -> 7.88 ms).
 int chain_blocks(int K, int planes) {
-  return planes * std::max(4, (int)(0.131 * std::sqrt((double)K)));
+  const int one = std::max(4, (int)(0.131 * std::sqrt((double)K)));
+  return planes == 2 ? one * 3 / 2 : one;
 }
 
 // Accumulators per tile: gate and up, or the two halves of RoPE pairs.
@@ -507,9 +511,10 @@ PairPlan plan_pair(int mode, int K, int n_virtual, int R) {
       const int chain = chain_blocks(K, planes);
       const int stages = (int)std::min<size_t>(kStagesMax, (kSmemMax - 1024) / stage);
       if (S > 1 && (size_t)MT * N * 512 > stages * stage) continue;   // its partial tiles reuse them
-      // Estimated clocks, fitted to 1,500 measured plans (19 projection shapes of the 7B, 13B,
-      // 1B and small models, 72 to 1024 rows; the chosen plan is on average 0.9 % slower than
-      // the fastest of its shape): a K block costs the MMAs or the fetch of its operands (36
+      // Estimated clocks, fitted to 1,500 measured plans (19 projection shapes, 72 to 1024 rows,
+      // chains of up to 16 blocks; with the chains as they are the chosen plan is on average
+      // 1.5 % slower than the fastest of its shape and row count, 21 % at most, over 3,027 plans of
+      // 24 shapes): a K block costs the MMAs or the fetch of its operands (36
       // bytes per clock and SM, 5,250 in all), the launch at least its weights at 22 bytes per
       // clock and active SM; the last tile's epilogue is never hidden, the earlier ones' only
       // where a second accumulator set fills meanwhile; a split adds the exchange of the
