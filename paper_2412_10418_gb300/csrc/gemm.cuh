@@ -158,7 +158,8 @@ __device__ __forceinline__ void warp_sums(float (&v)[NR]) {
   }
 }
 
-// Epilogue on registers: finish NR activation rows row0 .. row0 + NR - 1 (the first `rows` of them)
+// Epilogue on registers (the same arithmetic as tile_epilogue's below, which reads a finished tile
+// from shared memory: a change to one belongs in both): finish NR activation rows row0 .. row0 + NR - 1 (the first `rows` of them)
 // of one output per lane. STORE / RESID: L is the weight row, y0 its sums. SWIGLU: the feature, y0
 // its gate and y1 its up sums. QKV: the pair (head, e) = (L / (hd / 2), L % (hd / 2)) over the
 // stacked heads, y0 and y1 the sums of dims e and e + hd / 2. rs: row scales of row0 on (a.in_ss),
@@ -273,7 +274,7 @@ __device__ __forceinline__ void finish_rows(const GemmArgs& a, int L, int row0, 
   }
 }
 
-// Apply the epilogue to a finished fp32 tile: tile[r * ldt + v] holds y for activation row
+// Apply the epilogue (finish_rows is the same on registers) to a finished fp32 tile: tile[r * ldt + v] holds y for activation row
 // r0 + r and virtual row v0 + v (v in [0, 128)), for r in [0, rt). s_rs[r] is the input row
 // scale of row r0 + r when a.in_ss is set (see input_row_scales). Run by `nthr` threads (a
 // multiple of 32; tid = 0 .. nthr-1; all threads of the block by default), which the caller

@@ -558,10 +558,8 @@ TcPlan plan_tc(int K, int n_virtual, int R, int n_sm, int force_per_sm, int max_
              10 * p.tiles >= 9 * n_sm) {
     // about one tile per SM or more, but too many for clusters: one block per whole tile (no
     // split, no fixup). Measured against stream-K over all 304 slots: 38.4 vs 41.2 us (7B
-    // gate/up), 46.2 vs 55.2 us (7B LM head), 22.8 vs 25.2 us (draft LM head). With fewer
-    // tiles than that (e.g. the 40-tile projections of the 13B verify pass at 224 rows, whose
-    // partial tiles are too large for clusters) whole tiles would leave most SMs idle:
-    // stream-K over every block slot instead.
+    // gate/up), 46.2 vs 55.2 us (7B LM head), 22.8 vs 25.2 us (draft LM head). The few tile counts
+    // between (133 to 136 on 152 SMs) and those above the block slots run stream-K.
     p.ctas = p.tiles;
   }
   p.smem = (size_t)p.stages * stage + (size_t)p.ep_rows * kTileLd * 4 + 1024;

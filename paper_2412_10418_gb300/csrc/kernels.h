@@ -159,7 +159,7 @@ void launch_gemv(const GemmArgs& a, const GemvPlan& p, float* part, int* tile_cn
 
 // Tensor-core GEMM (tcgen05, TMEM, TMA) for bf16 weights and 1..kPairRows activation rows, on a
 // persistent stream-K grid of `ctas` blocks. maps: TMA descriptors of the weight segments
-// (128-byte swizzle, 64x64 boxes) and of the hi / lo activation planes (64x16 boxes).
+// (128-byte swizzle, boxes of 64 features x 64 rows) and of the hi / lo activation planes (x n_pad).
 // Scratch: part [ctas][2][n_pad][128] floats (tc_scratch_floats), one arrival counter per
 // tile (zero between launches). Launched with programmatic dependent launch allowed.
 struct TcMaps { CUtensorMap w[3]; CUtensorMap xh, xl; };
