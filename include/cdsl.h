@@ -90,9 +90,9 @@ typedef struct cdsl_run_cfg {
   float r_t;            /* reward threshold */
   int32_t reward_head;  /* 0: R = coverage; 1: R = 0.5 coverage + 0.5 sigmoid(w . h_last) */
   int32_t page_size;    /* KV page size in tokens (power of two, 16..256); 0 = 64 */
-  int32_t max_chunk;    /* rows per prefill forward pass; 0 = 1024 (or batch x max_prompt if less). The
-                         * workspace's activation buffers grow with it: 230 KB per row at 13B, 0 for
-                         * 256 takes 170 MB less of it */
+  int32_t max_chunk;    /* rows per prefill forward pass, at most batch x max_prompt; 0 = 1024. The
+                         * workspace grows with it (13B shapes: 209 KB per row, 160 MB from 256 to
+                         * 1024 rows); cdsl_workspace_size says by how much */
   /* Validation of the lookahead by M_p (Sec. 3.2.2):
    *   0: hard rejection: x_j is accepted while argmax p_j == x_j;
    *   1: speculative sampling: x_j is accepted while u_j <= min(1, p_j(x_j) / q_j(x_j)),

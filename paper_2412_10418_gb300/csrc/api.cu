@@ -222,7 +222,8 @@ void derive_dims(cdsl_ctx* c) {
   // weight is streamed once per 1024 prompt tokens, and a pass's launches and the wait that ends
   // it are shared by as many tokens (measured, prefill and first step: 32 small-model prompts
   // 14.3 ms at 256 rows, 9.7 at 512, 7.5 at 1024, 6.6 at 2048; 13B two-layer, 3,500 tokens
-  // 19.8, 17.6, 15.2, 13.7; the activation buffers grow with it, 170 MB of a 13B workspace)
+  // 19.8, 17.6, 15.2, 13.7, before the chains of its GEMMs were bounded; the activation buffers
+  // grow with it, 160 MB of a 13B workspace)
   const int chunk = r.max_chunk ? r.max_chunk : 1024;
   c->R_p = std::min(chunk, c->B * r.max_prompt);
   c->R_max = std::max(std::max(c->R_v, c->R_s1), std::max(c->R_d, c->R_p));
